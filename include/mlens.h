@@ -105,11 +105,11 @@ int mlens_set_precision(mlens_ctx *ctx, int32_t precision);
  * mlens_set_tuning -- launch shape of the FP32 kernels for later calls on this
  * context: rays_per_thread in {4, 8} (tile 64 x 16 or 64 x 32 rays per CTA of
  * 256 threads), star_stage in {128, 256, 512} stars staged through shared
- * memory at a time (0 = 256), and fma_pairs in {0, 1}: 0 takes every
+ * memory at a time (0 = 256; 512 is accepted and staged as 256), and fma_pairs in {0, 1}: 0 takes every
  * reciprocal 1/r^2 from the MUFU unit (16 per SM per clock, the bound of the
  * direct sum); 1 takes a share of them (a thread's first ray pair on every third
  * star, 7.8 %) from Newton-Raphson iterations on the FMA pipe instead, which
- * balances the two units (4.84e12 against 4.67e12 interactions/s on GB300).  The
+ * balances the two units (5.08e12 against 4.77e12 interactions/s on GB300).  The
  * stage size never changes the arithmetic; the tile shape (it moves the tile
  * centres) and the reciprocal source change beta in its last bits (never by
  * more than the error bar).  A given setting is deterministic.  Defaults: 8,
@@ -381,7 +381,7 @@ int mlens_batch_set_tuning(mlens_batch *b, int32_t rays_per_thread, int32_t star
 
 /*
  * mlens_batch_tune -- the autotuner: time the launch shapes (rays per thread 8
- * or 4, star stage 256 or 512, fma_pairs 0 or 1) on this batch (a warm-up and
+ * or 4, star stage 256 or 128, fma_pairs 0 or 1) on this batch (a warm-up and
  * two timed replays each, CUDA events on `stream`), keep the fastest and report
  * it (any output pointer may be NULL; *best_ms = -1 when the shape came from the
  * cache).  Results are cached per process by device and workload

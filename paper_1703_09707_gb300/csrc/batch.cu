@@ -330,7 +330,7 @@ int mlens_batch_tune(mlens_batch *b, void *stream, int32_t *rays_per_thread, int
         }
     }
     const int cand_rpt[2] = {8, 4};
-    const int cand_st[2] = {256, 512};
+    const int cand_st[2] = {256, 128};
     cudaEvent_t e0, e1;
     BCUDA(cudaEventCreate(&e0), "cudaEventCreate");
     BCUDA(cudaEventCreate(&e1), "cudaEventCreate");

@@ -1281,13 +1281,14 @@ constexpr int kNearChunk = NET ? 4 : 2;
 constexpr int kTcChunk = 128;                            // rays per tensor-core MMA (M)
 constexpr int kTcABytes = kTcChunk * kHid * 2;           // one warpgroup's A operand (16 KB)
 constexpr int kTcSmem = 2 * kTcABytes;                   // the two A operands
-constexpr size_t kLearnedDynSmem = kTcSmem > sizeof(ShootSmem<256>) ? kTcSmem : sizeof(ShootSmem<256>);
+using LearnTileSmem = ShootSmem<4, 256, true>;           // the near-field star stage, then the window
+constexpr size_t kLearnedDynSmem = kTcSmem > sizeof(LearnTileSmem) ? kTcSmem : sizeof(LearnTileSmem);
 
 // LO: the ray offsets carry low parts (grids whose offsets are not exact floats,
 // RayGrid lo); a separate instance so that the exact-offset tiles keep their
 // registers.
 template <bool NET, bool LO>
-__device__ __forceinline__ void learned_tile(const LearnedArgs &L, int bx, int by, ShootSmem<256> &sm, TileShared &ts,
+__device__ __forceinline__ void learned_tile(const LearnedArgs &L, int bx, int by, LearnTileSmem &sm, TileShared &ts,
                                              LearnSmem &ls, unsigned char *abuf_all, uint32_t &phase)
 {
     constexpr int NP = 4;
@@ -1644,7 +1645,7 @@ __device__ __forceinline__ void learned_tile(const LearnedArgs &L, int bx, int b
 // NET: the network on the tensor cores (tcgen05; 128 tensor-memory columns and the
 // two A operands in dynamic shared memory, in the same bytes as the star stage and
 // window); without it (the series alone) the kernel carries no tensor-core code.
-template <int NRP, bool NET, bool LO>
+template <bool NET, bool LO>
 // Four CTAs per SM (64 registers, ~280 bytes of spills per thread; tensor memory
 // holds four CTAs' 128 columns): eight warps per scheduler hide the latency of the
 // 128 hardware tanh per ray.  Measured per 32768^2-ray map: two CTAs per SM 0.060 s,
@@ -1658,7 +1659,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_shoot_learned(LearnedArgs L)
     // dynamic: the star stage and window of the tile phases without tensor-core work,
     // and (NET) the two A operands of the network phase in the same bytes
     extern __shared__ __align__(128) unsigned char dyn_smem[];
-    ShootSmem<256> &sm = *reinterpret_cast<ShootSmem<256> *>(dyn_smem);
+    LearnTileSmem &sm = *reinterpret_cast<LearnTileSmem *>(dyn_smem);
     unsigned char *tc_abuf = dyn_smem;
     const int tid = threadIdx.x;
     uint32_t phase = 0;  // completed MMA batches of this thread's warpgroup, mod 2
@@ -1688,11 +1689,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_shoot_learned(LearnedArgs L)
         if (item >= L.nitems) break;
         const int tile = L.items[item];
         const int bx = tile % ntx, by = tile / ntx;
-        const int rc = (by / L.cg.kty) * L.cg.ncx + bx / L.cg.ktx;
-        if (L.flags[rc])
-            shoot_tile<4, 256, false, NRP, 1, LO ? 2 : 1>(L.plain, bx, by, sm, ts);
-        else
-            learned_tile<NET, LO>(L, bx, by, sm, ts, ls, tc_abuf, phase);
+        learned_tile<NET, LO>(L, bx, by, sm, ts, ls, tc_abuf, phase);
     }
     if (NET) {
         // a warpgroup that gave up on a wait drains its MMAs (again bounded) before
@@ -1703,18 +1700,6 @@ __global__ void __launch_bounds__(kThreads, 4) k_shoot_learned(LearnedArgs L)
         umma::fence_after();
         if (tid < 32) umma::tmem_dealloc(ls.tmem, 2 * kHid);
     }
-}
-
-// Dynamic shared memory for the tensor-core operands, and the largest shared-memory
-// carveout for three CTAs of ~60 KB per SM.
-template <class K>
-static cudaError_t learned_attributes(K kernel)
-{
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLearnedDynSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared);
-    return e;
 }
 
 static_assert(kNetPairs * 2 == kHid, "NetConsts holds one entry per pair of hidden units");
@@ -1740,14 +1725,10 @@ cudaError_t ff_learned_grid(int *grid)
     // tensor-core variant has the same register limit and fits four CTAs in shared
     // and tensor memory, though the occupancy query has reported fewer for it; CTAs
     // beyond those resident only find the shared work queue empty.
-    int per_sm = 0, per_sm1 = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_shoot_learned<0, false, false>, kThreads,
-                                                                  sizeof(ShootSmem<256>));
+    int per_sm = 0;
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_shoot_learned<false, false>, kThreads,
+                                                                  sizeof(LearnTileSmem));
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm1, k_shoot_learned<1, false, false>, kThreads,
-                                                      sizeof(ShootSmem<256>));
-    if (e != cudaSuccess) return e;
-    per_sm = per_sm < per_sm1 ? per_sm : per_sm1;
     int dev = 0, nsm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -1755,29 +1736,23 @@ cudaError_t ff_learned_grid(int *grid)
     return cudaSuccess;
 }
 
-template <int NRP, bool LO>
+template <bool LO>
 static cudaError_t launch_learned_t(const LearnedArgs &L, unsigned g, cudaStream_t s)
 {
     if (L.use_net) {
-        cudaError_t e = learned_attributes(k_shoot_learned<NRP, true, LO>);
+        cudaError_t e = allow_dynamic_smem(k_shoot_learned<true, LO>, kLearnedDynSmem);
         if (e != cudaSuccess) return e;
-        k_shoot_learned<NRP, true, LO><<<g, kThreads, kLearnedDynSmem, s>>>(L);
+        k_shoot_learned<true, LO><<<g, kThreads, kLearnedDynSmem, s>>>(L);
     } else {
-        k_shoot_learned<NRP, false, LO><<<g, kThreads, sizeof(ShootSmem<256>), s>>>(L);
+        k_shoot_learned<false, LO><<<g, kThreads, sizeof(LearnTileSmem), s>>>(L);
     }
     return cudaGetLastError();
 }
 
-template <int NRP>
-static cudaError_t launch_learned(const LearnedArgs &L, unsigned g, cudaStream_t s)
+cudaError_t ff_shoot_learned(const LearnedArgs &L, int grid, cudaStream_t s)
 {
-    return L.plain.rays.lo ? launch_learned_t<NRP, true>(L, g, s) : launch_learned_t<NRP, false>(L, g, s);
-}
-
-cudaError_t ff_shoot_learned(const LearnedArgs &L, int grid, int fma_pairs, cudaStream_t s)
-{
-    const int64_t g = L.nitems < grid ? (L.nitems > 0 ? L.nitems : 1) : grid;
-    return fma_pairs ? launch_learned<1>(L, (unsigned)g, s) : launch_learned<0>(L, (unsigned)g, s);
+    const unsigned g = (unsigned)(L.nitems < grid ? (L.nitems > 0 ? L.nitems : 1) : grid);
+    return L.plain.rays.lo ? launch_learned_t<true>(L, g, s) : launch_learned_t<false>(L, g, s);
 }
 
 }  // namespace mlens

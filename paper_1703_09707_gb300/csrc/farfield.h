@@ -54,19 +54,18 @@ struct NetConsts {
 
 // Everything the learned shooting kernel reads.
 struct LearnedArgs {
-    ShootArgs plain;           // all stars, grids, counts, counters: used by fallback tiles and the epilogue
+    ShootArgs plain;           // grids, lens terms, counts, counters
     CellGrid cg;
     const int *cstart;         // extended cells + 1: CSR offsets into cstars
     const float4 *cstars;      // stars sorted by extended cell (input order within a cell)
     const float *coef;         // per ray cell kCoefStride floats
     const float *sc;           // per ray cell residual bound s_c
-    const int *flags;          // per ray cell: 1 = fall back to the plain sum
     const float *ec;           // per ray cell 64 floats: bf16(W1z) bf16(z_c) + b1
     const float *params;       // FP32 network parameters (flat layout of mlp.cuh)
     const __nv_bfloat16 *w2b;  // W2 in BF16, [out][in]
     int pe;
     int use_net;
-    const int *items;          // tile index per work item (fallback tiles first)
+    const int *items;          // tile index per work item (tiles of cells that passed validation)
     int64_t nitems;
     unsigned long long *counter;
     int *err;                  // set to 1 if a tensor-core completion wait gave up (results invalid)
@@ -153,8 +152,7 @@ int64_t ff_train_blocks(int64_t nsamples);  // CTAs of one ff_train_step
 cudaError_t ff_reduce_grads(const float *gpart, int64_t nblk, float *grads, float *loss, cudaStream_t s);
 cudaError_t ff_embed(const float *params, const float *z, int nrc, float *ec, cudaStream_t s);
 cudaError_t ff_flags(const unsigned *maxerr, int nrc, float tol, int *flags, cudaStream_t s);
-// fallback tiles use the plain tile function with the context's fma_pairs setting
-cudaError_t ff_shoot_learned(const LearnedArgs &L, int grid, int fma_pairs, cudaStream_t s);
+cudaError_t ff_shoot_learned(const LearnedArgs &L, int grid, cudaStream_t s);
 cudaError_t ff_learned_grid(int *grid);
 // The learned kernel's NetConsts from the flat FP32 parameters (host copy).
 void ff_net_consts(const float *params_host, NetConsts *out);

@@ -509,7 +509,6 @@ int mlens_shoot_learned(mlens_ctx *ctx, const mlens_grid *rays, const mlens_grid
     L.cstars = f->cstars;
     L.coef = f->coef;
     L.sc = f->sc;
-    L.flags = f->flags;
     L.ec = f->ec;
     L.params = f->params;
     L.w2b = f->w2b;
@@ -522,15 +521,13 @@ int mlens_shoot_learned(mlens_ctx *ctx, const mlens_grid *rays, const mlens_grid
     L.wait_probe = g_wait_probe.load();
     L.net = f->net;
     // Fallback tiles (each a full plain tile over all stars) run first, each split
-    // over a cluster of CTAs so that a few flagged cells do not set the map's
+    // over a cluster of CTAs where there are stars enough, so that a few flagged cells do not set the map's
     // time; the persistent learned kernel then takes the learned tiles.
-    const int split = fallback_star_split(ctx->n_pad);
-    if (split > 1 && nheavy > 0) {
-        FCUDA(launch_shoot_split_list(L.plain, items, nheavy, split, s, ctx->fma_pairs), "fallback tiles launch");
-        L.items = items + nheavy;
-        L.nitems = nitems - nheavy;
-    }
-    if (L.nitems > 0) FCUDA(ff_shoot_learned(L, f->grid, ctx->fma_pairs, s), "learned shoot launch");
+    FCUDA(launch_shoot_split_list(L.plain, items, nheavy, fallback_star_split(ctx->n_pad), s, ctx->fma_pairs),
+          "fallback tiles launch");
+    L.items = items + nheavy;
+    L.nitems = nitems - nheavy;
+    if (L.nitems > 0) FCUDA(ff_shoot_learned(L, f->grid, s), "learned shoot launch");
     if (stats_host) {
         unsigned long long h[3];
         int err = 0;

@@ -84,8 +84,20 @@ struct BatchLaunch {
     unsigned long long *counter;  // work-queue counter, zero before each launch (device)
 };
 
+// Let a kernel take `bytes` of dynamic shared memory, with the largest shared-memory
+// carveout of the SM (two CTAs of up to ~110 KB).
+template <class K>
+inline cudaError_t allow_dynamic_smem(K kernel, size_t bytes)
+{
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutMaxShared);
+    return e;
+}
+
 // launchers (defined in the .cu files)
-// pairs_per_thread in {2, 4} (4 or 8 rays per thread); stage in {128, 256, 512} stars
+// pairs_per_thread in {2, 4} (4 or 8 rays per thread); stage in {128, 256, 512} stars (512 runs as 256)
 // fma_pairs in {0, 1}: 1 takes a share of the reciprocals (pair 0 on every third
 // star, 7.8 %) from the FMA pipe, 0 every reciprocal from the MUFU unit
 // [ty0, ty1): the tile rows to shoot (tile_rows(pairs_per_thread) ray rows each;

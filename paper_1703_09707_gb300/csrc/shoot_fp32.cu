@@ -5,13 +5,14 @@
 //
 // One CTA of 256 threads owns a 64 x (8*NP) tile of the ray grid; each thread
 // owns 2*NP rays of one grid column, processed as NP packed pairs with the
-// Blackwell f32x2 instructions (FADD2/FMUL2/FFMA2), so one instruction serves
-// two rays.  Stars stream through shared memory in stages of SC; each stage is
-// re-centred on the tile (star minus tile centre, once per star per CTA) and
-// stored duplicated as (-dx,-dx,-dy,-dy),(m,m) so that a single broadcast
-// LDS.128 + LDS.64 feeds every packed pair.  Per star and ray the work is
-// FADD, FFMA (r^2), MUFU.RCP, FMUL (m/r^2), 2 FFMA (accumulate): the MUFU
-// reciprocal (16 per SM per clock) is the only unit near saturation.
+// Blackwell f32x2 instructions (FMUL2/FFMA2), so one instruction serves two rays.
+// Stars stream through shared memory in stages of SC; a stage holds, per star, the
+// differences y_ray - y_star of the tile's rows, the mass and the re-centred x
+// (tile.cuh RowStage), read as broadcasts.  Per star and ray the work is FFMA (r^2),
+// MUFU.RCP, FMUL (m/r^2), 2 FFMA (accumulate): the MUFU reciprocal (16 per SM per
+// clock) is the unit nearest saturation (shoot_tile has the count of both pipes).
+// A stage of SC = 256 stars is 74 KB (NP = 4): two CTAs per SM.  The API's stage of
+// 512 runs as 256: 147 KB would leave one CTA per SM.
 //
 // Precision (MLENS_PREC_FP32): rays and stars are relative to an FP32 tile
 // centre c, so differences of nearby positions carry no absolute-coordinate
@@ -37,9 +38,10 @@ namespace mlens {
 template <int NP, int SC, bool NAIVE, int NRP>
 __global__ void __launch_bounds__(kThreads, 2) k_shoot_fp32(ShootArgs a, int by0)
 {
-    __shared__ __align__(16) ShootSmem<SC> sm;
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
     __shared__ TileShared ts;
-    shoot_tile<NP, SC, NAIVE, NRP>(a, blockIdx.x, by0 + (int)blockIdx.y, sm, ts);
+    shoot_tile<NP, SC, NAIVE, NRP>(a, blockIdx.x, by0 + (int)blockIdx.y,
+                                   *reinterpret_cast<ShootSmem<NP, SC, NAIVE> *>(dyn_smem), ts);
 }
 
 // Persistent kernel over many fields: CTAs pull (field, tile) items from one
@@ -51,7 +53,8 @@ __global__ void __launch_bounds__(kThreads, 2)
     k_shoot_batch(const ShootArgs *fields, const int *order, const int64_t *begin, int nf, int64_t total,
                   unsigned long long *counter)
 {
-    __shared__ __align__(16) ShootSmem<SC> sm;
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    ShootSmem<NP, SC> &sm = *reinterpret_cast<ShootSmem<NP, SC> *>(dyn_smem);
     __shared__ TileShared ts;
     __shared__ long long s_item;
     for (;;) {
@@ -85,10 +88,13 @@ static cudaError_t launch_t(const ShootArgs &a, cudaStream_t s, int ty0, int ty1
 {
     // tile rows in launches of at most 65535 (the grid's y limit)
     const int tx = (a.rays.nx + kTileX - 1) / kTileX, ty = tile_row_end(a, NP, ty1);
+    constexpr size_t smem = sizeof(ShootSmem<NP, SC, NAIVE>);
+    cudaError_t e = allow_dynamic_smem(k_shoot_fp32<NP, SC, NAIVE, NRP>, smem);
+    if (e != cudaSuccess) return e;
     for (int by0 = ty0; by0 < ty; by0 += 65535) {
         const dim3 grid((unsigned)tx, (unsigned)min(65535, ty - by0));
-        k_shoot_fp32<NP, SC, NAIVE, NRP><<<grid, kThreads, 0, s>>>(a, by0);
-        const cudaError_t e = cudaGetLastError();
+        k_shoot_fp32<NP, SC, NAIVE, NRP><<<grid, kThreads, smem, s>>>(a, by0);
+        e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -99,11 +105,9 @@ static cudaError_t launch_sel(const ShootArgs &a, int np, int sc, cudaStream_t s
 {
     if (np == 2) {
         if (sc == 128) return launch_t<2, 128, NAIVE, NRP>(a, s, ty0, ty1);
-        if (sc == 512) return launch_t<2, 512, NAIVE, NRP>(a, s, ty0, ty1);
         return launch_t<2, 256, NAIVE, NRP>(a, s, ty0, ty1);
     }
     if (sc == 128) return launch_t<4, 128, NAIVE, NRP>(a, s, ty0, ty1);
-    if (sc == 512) return launch_t<4, 512, NAIVE, NRP>(a, s, ty0, ty1);
     return launch_t<4, 256, NAIVE, NRP>(a, s, ty0, ty1);
 }
 
@@ -125,7 +129,10 @@ template <int NP, int SC, int NRP>
 static cudaError_t grid_b(int *grid)
 {
     int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_shoot_batch<NP, SC, NRP>, kThreads, 0);
+    constexpr size_t smem = sizeof(ShootSmem<NP, SC>);
+    cudaError_t e = allow_dynamic_smem(k_shoot_batch<NP, SC, NRP>, smem);
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_shoot_batch<NP, SC, NRP>, kThreads, smem);
     if (e != cudaSuccess) return e;
     int dev = 0, nsm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -139,11 +146,9 @@ static cudaError_t grid_sel(int np, int sc, int *grid)
 {
     if (np == 2) {
         if (sc == 128) return grid_b<2, 128, NRP>(grid);
-        if (sc == 512) return grid_b<2, 512, NRP>(grid);
         return grid_b<2, 256, NRP>(grid);
     }
     if (sc == 128) return grid_b<4, 128, NRP>(grid);
-    if (sc == 512) return grid_b<4, 512, NRP>(grid);
     return grid_b<4, 256, NRP>(grid);
 }
 
@@ -157,7 +162,10 @@ static cudaError_t launch_b(const BatchLaunch &b, cudaStream_t s)
 {
     const int64_t want = b.grid > 0 ? b.grid : 1;
     const unsigned grid = (unsigned)(b.total < want ? (b.total > 0 ? b.total : 1) : want);
-    k_shoot_batch<NP, SC, NRP><<<grid, kThreads, 0, s>>>(b.fields, b.order, b.begin, b.nfields, b.total, b.counter);
+    constexpr size_t smem = sizeof(ShootSmem<NP, SC>);
+    const cudaError_t e = allow_dynamic_smem(k_shoot_batch<NP, SC, NRP>, smem);
+    if (e != cudaSuccess) return e;
+    k_shoot_batch<NP, SC, NRP><<<grid, kThreads, smem, s>>>(b.fields, b.order, b.begin, b.nfields, b.total, b.counter);
     return cudaGetLastError();
 }
 
@@ -166,11 +174,9 @@ static cudaError_t launch_bsel(const BatchLaunch &b, int np, int sc, cudaStream_
 {
     if (np == 2) {
         if (sc == 128) return launch_b<2, 128, NRP>(b, s);
-        if (sc == 512) return launch_b<2, 512, NRP>(b, s);
         return launch_b<2, 256, NRP>(b, s);
     }
     if (sc == 128) return launch_b<4, 128, NRP>(b, s);
-    if (sc == 512) return launch_b<4, 512, NRP>(b, s);
     return launch_b<4, 256, NRP>(b, s);
 }
 

@@ -24,15 +24,18 @@ static inline int tile_row_end_s(const ShootArgs &a, int np, int ty1)
     return ty1 < 0 || ty1 > ty ? ty : ty1;
 }
 
+template <int NP>
+using SplitSmem = ShootSmem<NP, kSplitStage>;
+
 // Split star sum: clusters of SPLIT CTAs along x share one tile (tile column
 // blockIdx.x / SPLIT); partials are reduced through distributed shared memory.
 template <int NP, int SPLIT, int NRP>
 __global__ void __launch_bounds__(kThreads, 2) k_shoot_split(ShootArgs a, int by0)
 {
-    __shared__ __align__(16) ShootSmem<kSplitStage> sm;
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
     __shared__ TileShared ts;
-    extern __shared__ float4 part[];  // 2 NP float4 per thread
-    shoot_tile<NP, kSplitStage, false, NRP, SPLIT>(a, (int)(blockIdx.x / SPLIT), by0 + (int)blockIdx.y, sm, ts, part);
+    shoot_tile<NP, kSplitStage, false, NRP, SPLIT>(a, (int)(blockIdx.x / SPLIT), by0 + (int)blockIdx.y,
+                                                   *reinterpret_cast<SplitSmem<NP> *>(dyn_smem), ts);
 }
 
 // Split star sum through global memory: CTA (tile column blockIdx.x / R, slice
@@ -41,11 +44,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_shoot_split(ShootArgs a, int by
 template <int NP, int NRP>
 __global__ void __launch_bounds__(kThreads, 2) k_shoot_slices(ShootArgs a, int by0, int ty_base)
 {
-    __shared__ __align__(16) ShootSmem<kSplitStage> sm;
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
     __shared__ TileShared ts;
     const int R = a.gslices, tiles_x = (a.rays.nx + kTileX - 1) / kTileX;
     const int bx = (int)(blockIdx.x / R), r = (int)(blockIdx.x % R), by = by0 + (int)blockIdx.y;
-    shoot_tile<NP, kSplitStage, false, NRP, 1, 0, 1>(a, bx, by, sm, ts, nullptr,
+    shoot_tile<NP, kSplitStage, false, NRP, 1, 0, 1>(a, bx, by, *reinterpret_cast<SplitSmem<NP> *>(dyn_smem), ts,
                                                       (int64_t)(by - ty_base) * tiles_x + bx, r);
 }
 
@@ -53,11 +56,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_shoot_slices(ShootArgs a, int b
 template <int NP>
 __global__ void __launch_bounds__(kThreads, 2) k_fold_slices(ShootArgs a, int by0, int ty_base)
 {
-    __shared__ __align__(16) ShootSmem<kSplitStage> sm;
+    __shared__ __align__(16) ShootSmem<NP, 32> sm;  // no stars are staged
     __shared__ TileShared ts;
     const int tiles_x = (a.rays.nx + kTileX - 1) / kTileX;
     const int bx = (int)blockIdx.x, by = by0 + (int)blockIdx.y;
-    shoot_tile<NP, kSplitStage, false, 0, 1, 0, 2>(a, bx, by, sm, ts, nullptr, (int64_t)(by - ty_base) * tiles_x + bx);
+    shoot_tile<NP, 32, false, 0, 1, 0, 2>(a, bx, by, sm, ts, (int64_t)(by - ty_base) * tiles_x + bx);
 }
 
 template <int NP, int SPLIT, int NRP>
@@ -71,15 +74,8 @@ static cudaError_t launch_split_t(const ShootArgs &a, cudaStream_t s, int ty0, i
     attr[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = 2 * NP * kThreads * sizeof(float4);
-    // static (the stage/window union) + dynamic (partials) exceeds the 48 KB a
-    // launch gets without opting in for NP = 4
-    cudaError_t e0 = cudaFuncSetAttribute(k_shoot_split<NP, SPLIT, NRP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)cfg.dynamicSmemBytes);
-    // two CTAs of ~49 KB per SM: ask for the largest shared-memory carveout
-    if (e0 == cudaSuccess)
-        e0 = cudaFuncSetAttribute(k_shoot_split<NP, SPLIT, NRP>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                  (int)cudaSharedmemCarveoutMaxShared);
+    cfg.dynamicSmemBytes = sizeof(SplitSmem<NP>);
+    const cudaError_t e0 = allow_dynamic_smem(k_shoot_split<NP, SPLIT, NRP>, cfg.dynamicSmemBytes);
     if (e0 != cudaSuccess) return e0;
     cfg.stream = s;
     cfg.attrs = attr;
@@ -92,17 +88,16 @@ static cudaError_t launch_split_t(const ShootArgs &a, cudaStream_t s, int ty0, i
     return cudaSuccess;
 }
 
-// The split star sum over a list of tiles (tile = by * tiles_x + bx), one
-// cluster per listed tile: the learned far field's fallback tiles.
+// The (split) star sum over a list of tiles (tile = by * tiles_x + bx), one cluster
+// (SPLIT = 1: one CTA) per listed tile: the learned far field's fallback tiles.
 template <int SPLIT, int NRP>
 __global__ void __launch_bounds__(kThreads, 2) k_shoot_split_list(ShootArgs a, const int *tiles)
 {
-    __shared__ __align__(16) ShootSmem<kSplitStage> sm;
+    extern __shared__ __align__(16) unsigned char dyn_smem[];
     __shared__ TileShared ts;
-    extern __shared__ float4 part[];  // 2 NP float4 per thread
     const int ntx = (a.rays.nx + kTileX - 1) / kTileX;
     const int t = tiles[blockIdx.x / SPLIT];
-    shoot_tile<4, kSplitStage, false, NRP, SPLIT>(a, t % ntx, t / ntx, sm, ts, part);
+    shoot_tile<4, kSplitStage, false, NRP, SPLIT>(a, t % ntx, t / ntx, *reinterpret_cast<SplitSmem<4> *>(dyn_smem), ts);
 }
 
 template <int SPLIT, int NRP>
@@ -115,15 +110,11 @@ static cudaError_t launch_split_list_t(const ShootArgs &a, const int *tiles, int
     attr[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = 2 * 4 * kThreads * sizeof(float4);
+    cfg.dynamicSmemBytes = sizeof(SplitSmem<4>);
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaFuncSetAttribute(k_shoot_split_list<SPLIT, NRP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)cfg.dynamicSmemBytes);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_shoot_split_list<SPLIT, NRP>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutMaxShared);
+    const cudaError_t e = allow_dynamic_smem(k_shoot_split_list<SPLIT, NRP>, cfg.dynamicSmemBytes);
     if (e != cudaSuccess) return e;
     cfg.gridDim = dim3((unsigned)(ntiles * SPLIT));
     return cudaLaunchKernelEx(&cfg, k_shoot_split_list<SPLIT, NRP>, a, tiles);
@@ -132,6 +123,7 @@ static cudaError_t launch_split_list_t(const ShootArgs &a, const int *tiles, int
 template <int NRP>
 static cudaError_t launch_split_list_r(const ShootArgs &a, const int *tiles, int64_t ntiles, int split, cudaStream_t s)
 {
+    if (split == 1) return launch_split_list_t<1, NRP>(a, tiles, ntiles, s);
     if (split == 2) return launch_split_list_t<2, NRP>(a, tiles, ntiles, s);
     if (split == 4) return launch_split_list_t<4, NRP>(a, tiles, ntiles, s);
     if (split == 8) return launch_split_list_t<8, NRP>(a, tiles, ntiles, s);
@@ -240,16 +232,15 @@ static cudaError_t launch_gsplit_t(const ShootArgs &a0, int split, float4 *part,
     a.gpart = part;
     a.gslices = split;
     const int tx = (a.rays.nx + kTileX - 1) / kTileX, ty = tile_row_end_s(a, NP, ty1);
-    // static shared memory only (two CTAs of ~17 KB per SM): the largest carveout
-    cudaError_t e = cudaFuncSetAttribute(k_shoot_slices<NP, NRP>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                         (int)cudaSharedmemCarveoutMaxShared);
+    constexpr size_t smem = sizeof(SplitSmem<NP>);
+    cudaError_t e = allow_dynamic_smem(k_shoot_slices<NP, NRP>, smem);
     if (e != cudaSuccess) return e;
     if ((int64_t)tx * split > 0x7fffffff) return cudaErrorInvalidConfiguration;
     // one pass per rows_per_pass tile rows: the slices, then their fold (same stream,
     // so the next pass's slices overwrite partials the fold has read)
     for (int by0 = ty0; by0 < ty; by0 += rows_per_pass) {
         const int rows = std::min(rows_per_pass, ty - by0);
-        k_shoot_slices<NP, NRP><<<dim3((unsigned)(tx * split), (unsigned)rows), kThreads, 0, s>>>(a, by0, by0);
+        k_shoot_slices<NP, NRP><<<dim3((unsigned)(tx * split), (unsigned)rows), kThreads, smem, s>>>(a, by0, by0);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         k_fold_slices<NP><<<dim3((unsigned)tx, (unsigned)rows), kThreads, 0, s>>>(a, by0, by0);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;

@@ -23,22 +23,42 @@ constexpr int kKahan = 32;                 // stars per compensated partial
 
 static_assert(kStarPad % kKahan == 0, "star padding must be whole Kahan chunks");
 
-template <int SC>
-struct StarStage {
-    float4 q[2][SC];   // (-dx, -dx, -dy, -dy) relative to the tile centre
-    float2 mm[2][SC];  // (m, m)
+// Shared memory of one tile: two star stages (double buffered), whose bytes then
+// hold the binning window.
+//
+// Re-centred kernels (RowStage): the y offsets ray - star of a tile depend only on
+// the ray's row and the star, so a stage holds them ready: per star the tile's 8 NP
+// row offsets, then (m, m, -dx, 0) relative to the tile centre.  A thread reads its
+// 2 NP rows' offsets as NP / 2 broadcast LDS.128 instead of forming them with NP
+// packed additions.  An odd number of float4 per star keeps the staging threads'
+// stores (one star each) free of bank conflicts.
+//
+// Naive kernel (StarStage): absolute coordinates, duplicated for packed arithmetic.
+template <int NP, int SC>
+struct RowStage {
+    static constexpr int kStride = 2 * NP + 1;  // float4 per star
+    float4 s[2][SC * kStride];
 };
 
 template <int SC>
+struct StarStage {
+    float4 q[2][SC];   // (-x, -x, -y, -y)
+    float2 mm[2][SC];  // (m, m)
+};
+
+template <int NP, int SC, bool NAIVE = false>
 union ShootSmem {
-    StarStage<SC> st;
+    std::conditional_t<NAIVE, StarStage<SC>, RowStage<NP, SC>> st;
     uint32_t hist[kWin * kWin];
 };
+
+constexpr int kMaxRows = 32;  // ray rows of the largest tile (NP = 4)
 
 struct TileShared {
     float tc[10];      // cx, cy, ex, ey, B0h.x, B0h.y, B0l.x, B0l.y, exl, eyl
     int win[2];
     unsigned sred[3];
+    __align__(16) float ro[kMaxRows], rl[kMaxRows];  // the rows' offsets from the tile centre: high, low parts
 };
 
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
@@ -120,17 +140,29 @@ __device__ __forceinline__ float2 rcp_nr2(float2 x)
 // stages, beta, binning, counters.  Every thread of the CTA must call it.
 // NRP = 1: ray pair 0 takes its reciprocals from rcp_nr2 (FMA pipe) on every third
 // star of a 32-star chunk (stars 2, 5, .., 29: 10 of the 128 reciprocals a thread
-// forms per chunk, 7.8 %); all others come from the MUFU unit.  That share
-// balances the two pipes best on GB300 (measured: 4.84e12 interactions/s against
-// 4.67e12 with MUFU alone, 4.79e12 at 1/8 and 4.39e12 at 1/4 of the reciprocals).
+// forms per chunk, 7.8 %); all others come from the MUFU unit.
 // NRP = 0: MUFU alone.
+//
+// What bounds the re-centred star loop, per star and warp (8 rays a thread) on one of
+// the SM's four schedulers: MUFU, 59 cycles (8 reciprocals of 8 cycles, less the
+// Newton share), against the FP32 pipe.  A packed FP32 operation holds the pipe for 2
+// cycles, and 3 when its three operands are all different register pairs (measured; the
+// operand ports deliver two 32-bit registers a cycle), which the accumulations
+// f dx + px and f dy + py are.  Forming dx, dx^2 and dy in packed form in every thread
+// put the FP32 pipe level with MUFU: 66.6 cycles a star, 138.8 ms for 1e4 stars x
+// 8192^2 rays.  dx and dx^2 are the same in both lanes, so scalar operations and a copy
+// replace the packed ones (135 ms); dy comes ready from the stage (RowStage): 132.2 ms,
+// 63.4 cycles a star, 0.93 of the MUFU bound, and on grids whose offsets carry low parts
+// 21.87 -> 18.49 ms (9999 stars x 3001 x 2999 rays), since dy's low part is added once
+// per row instead of once per ray.  More warps per SM (80 or 64 registers, the Kahan
+// sums in shared memory) ran slower (145 ms): spills, and the same two pipes.
 //
 // SPLIT > 1 (re-centred FP32 only): the CTA is rank r of a cluster of SPLIT CTAs
 // that share the tile; it sums the r-th of SPLIT consecutive 32-aligned slices
-// of the stars.  Ranks 1.. leave their (S, C) partials in `part` (2 NP float4
-// per thread, in their own shared memory); rank 0 reads them through
-// distributed shared memory in rank order, folds each in with two Kahan steps
-// (S_r, then -C_r) and alone goes on to beta and binning.
+// of the stars.  Ranks 1.. leave their (S, C) partials in their own stage memory
+// (2 NP float4 per thread); rank 0 reads them through distributed shared memory in
+// rank order, folds each in with two Kahan steps (S_r, then -C_r) and alone goes on
+// to beta and binning.
 // LOM: how the tile learns whether the ray offsets need low parts: 0 = from the grid
 // at run time (RayGrid lo, both loops compiled), 1 = never, 2 = always (callers
 // that have chosen already).
@@ -143,13 +175,14 @@ __device__ __forceinline__ float2 rcp_nr2(float2 x)
 // as its own, folds the others in slice order (two Kahan steps each, S_r then -C_r,
 // as the cluster fold does) and goes on to beta and binning.
 template <int NP, int SC, bool NAIVE, int NRP = 0, int SPLIT = 1, int LOM = 0, int GS = 0>
-__device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, ShootSmem<SC> &sm, TileShared &ts,
-                                           float4 *part = nullptr, int64_t gtile = 0, int gslice = 0)
+__device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, ShootSmem<NP, SC, NAIVE> &sm,
+                                           TileShared &ts, int64_t gtile = 0, int gslice = 0)
 {
     static_assert(SPLIT == 1 || !NAIVE, "the split sum is for the re-centred kernel");
     static_assert(GS == 0 || (!NAIVE && SPLIT == 1), "the global split is for the re-centred kernel");
+    static_assert(SC <= kThreads, "one thread stages one star");
     constexpr int kTileY = tile_rows(NP);
-    constexpr int kLoads = (SC + kThreads - 1) / kThreads;
+    static_assert(kTileY <= kMaxRows, "TileShared holds the tile's rows");
     const int tid = threadIdx.x;
     const int tx = tid % kTileX;
     const int tg = tid / kTileX;
@@ -185,62 +218,30 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
     __syncthreads();
 
     // ------------------------------------------------------- this thread's rays
-    float2 rx;       // packed (x, x): both rays of a pair share the column
-    float2 ry[NP];   // packed (y_2p, y_2p+1)
-    float2 rxl, ryl[NP];               // low parts of the offsets (re-centred variants)
+    float rxh = 0.f, rxl = 0.f;        // the column's offset from the tile centre (NAIVE: its coordinate): high, low part
     float2 px[NP], py[NP];             // partial sums (NAIVE: the whole running sum)
     float2 Sx[NP], Sy[NP], Cx[NP], Cy[NP];
     const float kx = (float)tx;
-    float cx = 0.f, cy = 0.f;
     const bool lo = !NAIVE && (LOM == 2 || (LOM == 0 && R.lo));
     if (!NAIVE) {
-        cx = ts.tc[0];
-        cy = ts.tc[1];
         if (lo) {
-            float h, l;
-            ray_offset(kx, ts.tc[2], ts.tc[8], R.dxh, R.dxl, h, l);
-            rx = f2(h, h);
-            rxl = f2(l, l);
-#pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                float k0 = (float)(tg * 2 * NP + 2 * p), k1 = k0 + 1.0f;
-                float h1, l1;
-                ray_offset(k0, ts.tc[3], ts.tc[9], R.dyh, R.dyl, h, l);
-                ray_offset(k1, ts.tc[3], ts.tc[9], R.dyh, R.dyl, h1, l1);
-                ry[p] = f2(h, h1);
-                ryl[p] = f2(l, l1);
-            }
+            ray_offset(kx, ts.tc[2], ts.tc[8], R.dxh, R.dxl, rxh, rxl);
         } else {
             // exact float offsets (RayGrid lo = 0): e + k d with every step exact
-            const float dxr = __fmaf_rn(kx, R.dxh, ts.tc[2]);
-            rx = f2(dxr, dxr);
-            rxl = f2(0.f, 0.f);
-#pragma unroll
-            for (int p = 0; p < NP; ++p) {
-                float k0 = (float)(tg * 2 * NP + 2 * p), k1 = k0 + 1.0f;
-                ry[p] = f2(__fmaf_rn(k0, R.dyh, ts.tc[3]), __fmaf_rn(k1, R.dyh, ts.tc[3]));
-                ryl[p] = f2(0.f, 0.f);
-            }
+            rxh = __fmaf_rn(kx, R.dxh, ts.tc[2]);
+        }
+        if (tid < kTileY) {  // the rows' offsets
+            float h, l = 0.0f;
+            if (lo) ray_offset((float)tid, ts.tc[3], ts.tc[9], R.dyh, R.dyl, h, l);
+            else h = __fmaf_rn((float)tid, R.dyh, ts.tc[3]);
+            ts.ro[tid] = h;
+            ts.rl[tid] = l;
         }
 #pragma unroll
         for (int p = 0; p < NP; ++p) px[p] = py[p] = Sx[p] = Sy[p] = Cx[p] = Cy[p] = f2(0.f, 0.f);
+        __syncthreads();
     } else {
-        const float x0f = (float)R.x0, y0f = (float)R.y0;
-        const float dxf = (float)R.dx, dyf = (float)R.dy;
-        float thx = x0f + ((float)(i0 + tx) + 0.5f) * dxf;
-        rx = f2(thx, thx);
-        rxl = f2(0.f, 0.f);
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            float y0 = y0f + ((float)(j0 + tg * 2 * NP + 2 * p) + 0.5f) * dyf;
-            float y1 = y0f + ((float)(j0 + tg * 2 * NP + 2 * p + 1) + 0.5f) * dyf;
-            ry[p] = f2(y0, y1);
-            ryl[p] = f2(0.f, 0.f);
-            // alpha_0 first (Algorithm 1), then every star is added to it
-            px[p] = f2(a.lens.fm11 * thx + a.lens.fm12 * y0, a.lens.fm11 * thx + a.lens.fm12 * y1);
-            py[p] = f2(a.lens.fm12 * thx + a.lens.fm22 * y0, a.lens.fm12 * thx + a.lens.fm22 * y1);
-            Sx[p] = Sy[p] = Cx[p] = Cy[p] = f2(0.f, 0.f);
-        }
+        rxh = (float)R.x0 + ((float)(i0 + tx) + 0.5f) * (float)R.dx;
     }
 
     // ---------------------------------------------------------- star stages
@@ -260,65 +261,118 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
     }
     if (GS == 2) nst = 0;
     const int nstage = (int)((nst + SC - 1) / SC);
-    float4 nxt[kLoads];
+    float4 nxt;
     auto stage_load = [&](int s) {
-        const int64_t base = (int64_t)s * SC;
-#pragma unroll
-        for (int l = 0; l < kLoads; ++l) {
-            const int k = tid + l * kThreads;
-            nxt[l] = (k < SC && base + k < nst) ? __ldg(&stars[base + k]) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        const int64_t k = (int64_t)s * SC + tid;
+        nxt = (tid < SC && k < nst) ? __ldg(&stars[k]) : make_float4(0.f, 0.f, 0.f, 0.f);
     };
-    auto stage_store = [&](int buf) {
+    if constexpr (NAIVE) {
+        const float y0f = (float)R.y0, dyf = (float)R.dy;
+        const float2 rx = f2(rxh, rxh);
+        float2 ry[NP];
 #pragma unroll
-        for (int l = 0; l < kLoads; ++l) {
-            const int k = tid + l * kThreads;
-            if (k < SC) {
-                const float4 q = nxt[l];
-                float nx = NAIVE ? -q.x : __fsub_rn(cx, q.x);
-                float ny = NAIVE ? -q.y : __fsub_rn(cy, q.y);
-                sm.st.q[buf][k] = make_float4(nx, nx, ny, ny);
-                sm.st.mm[buf][k] = f2(q.z, q.z);
+        for (int p = 0; p < NP; ++p) {
+            const float y0 = y0f + ((float)(j0 + tg * 2 * NP + 2 * p) + 0.5f) * dyf;
+            const float y1 = y0f + ((float)(j0 + tg * 2 * NP + 2 * p + 1) + 0.5f) * dyf;
+            ry[p] = f2(y0, y1);
+            // alpha_0 first (Algorithm 1), then every star is added to it
+            px[p] = f2(a.lens.fm11 * rxh + a.lens.fm12 * y0, a.lens.fm11 * rxh + a.lens.fm12 * y1);
+            py[p] = f2(a.lens.fm12 * rxh + a.lens.fm22 * y0, a.lens.fm12 * rxh + a.lens.fm22 * y1);
+        }
+        auto stage_store = [&](int buf) {
+            if (tid < SC) {
+                sm.st.q[buf][tid] = make_float4(-nxt.x, -nxt.x, -nxt.y, -nxt.y);
+                sm.st.mm[buf][tid] = f2(nxt.z, nxt.z);
             }
+        };
+        if (nstage > 0) {
+            stage_load(0);
+            stage_store(0);
         }
-    };
-    if (nstage > 0) {
-        stage_load(0);
-        stage_store(0);
-    }
-    __syncthreads();
-
-    for (int s = 0; s < nstage; ++s) {
-        const int buf = s & 1;
-        const int cnt = (int)min((int64_t)SC, nst - (int64_t)s * SC);
-        if (s + 1 < nstage) stage_load(s + 1);
-        const float4 *Q = sm.st.q[buf];
-        const float2 *M = sm.st.mm[buf];
-        // the chunks of the stage; LO: the offsets' low parts are added after the
-        // subtraction (grids whose ray offsets are not exact floats, RayGrid lo)
-        auto chunks = [&](auto lo_tag) {
-            constexpr bool LO = decltype(lo_tag)::value && !NAIVE;
+        __syncthreads();
+        for (int s = 0; s < nstage; ++s) {
+            const int buf = s & 1;
+            const int cnt = (int)min((int64_t)SC, nst - (int64_t)s * SC);
+            if (s + 1 < nstage) stage_load(s + 1);
+            const float4 *Q = sm.st.q[buf];
+            const float2 *M = sm.st.mm[buf];
 #pragma unroll 1
             for (int k0 = 0; k0 < cnt; k0 += kKahan) {
 #pragma unroll
                 for (int k = k0; k < k0 + kKahan; ++k) {
                     const float4 q = Q[k];
                     const float2 m2 = M[k];
-                    const float2 dx = LO ? __fadd2_rn(__fadd2_rn(rx, f2(q.x, q.y)), rxl) : __fadd2_rn(rx, f2(q.x, q.y));
+                    const float2 dx = __fadd2_rn(rx, f2(q.x, q.y));
                     const float2 dx2 = __fmul2_rn(dx, dx);
                     const float2 nyv = f2(q.z, q.w);
 #pragma unroll
                     for (int p = 0; p < NP; ++p) {
-                        const float2 dy = LO ? __fadd2_rn(__fadd2_rn(ry[p], nyv), ryl[p]) : __fadd2_rn(ry[p], nyv);
+                        const float2 dy = __fadd2_rn(ry[p], nyv);
                         const float2 r2 = __ffma2_rn(dy, dy, dx2);
-                        const float2 inv = NRP > 0 && p == 0 && (k - k0) % 3 == 2 ? rcp_nr2(r2)
-                                                                                 : f2(rcp_approx(r2.x), rcp_approx(r2.y));
-                        const float2 f = __fmul2_rn(m2, inv);
+                        const float2 f = __fmul2_rn(m2, f2(rcp_approx(r2.x), rcp_approx(r2.y)));
                         px[p] = __ffma2_rn(f, dx, px[p]);
                         py[p] = __ffma2_rn(f, dy, py[p]);
                     }
                 }
-                if (!NAIVE) {
+            }
+            if (s + 1 < nstage) stage_store(buf ^ 1);
+            __syncthreads();
+        }
+    } else {
+        constexpr int kStride = RowStage<NP, SC>::kStride;
+        auto stage_store = [&](int buf) {  // thread t: star t against every row of the tile
+            if (tid >= SC) return;
+            const float ny = __fsub_rn(ts.tc[1], nxt.y);
+            float4 *dst = sm.st.s[buf] + tid * kStride;
+#pragma unroll
+            for (int r = 0; r < kTileY / 4; ++r) {
+                const float4 o = reinterpret_cast<const float4 *>(ts.ro)[r];
+                float4 d = make_float4(__fadd_rn(o.x, ny), __fadd_rn(o.y, ny), __fadd_rn(o.z, ny), __fadd_rn(o.w, ny));
+                if (lo) {  // after the subtraction of the star's offset (ray_offset)
+                    const float4 l = reinterpret_cast<const float4 *>(ts.rl)[r];
+                    d = make_float4(__fadd_rn(d.x, l.x), __fadd_rn(d.y, l.y), __fadd_rn(d.z, l.z), __fadd_rn(d.w, l.w));
+                }
+                dst[r] = d;
+            }
+            dst[kTileY / 4] = make_float4(nxt.z, nxt.z, __fsub_rn(ts.tc[0], nxt.x), 0.0f);
+        };
+        if (nstage > 0) {
+            stage_load(0);
+            stage_store(0);
+        }
+        __syncthreads();
+        for (int s = 0; s < nstage; ++s) {
+            const int buf = s & 1;
+            const int cnt = (int)min((int64_t)SC, nst - (int64_t)s * SC);
+            if (s + 1 < nstage) stage_load(s + 1);
+            // the chunks of the stage; LO: the column's low part is added after the
+            // subtraction (grids whose ray offsets are not exact floats, RayGrid lo)
+            auto chunks = [&](auto lo_tag) {
+                constexpr bool LO = decltype(lo_tag)::value;
+#pragma unroll 1
+                for (int k0 = 0; k0 < cnt; k0 += kKahan) {
+                    const float4 *Q = sm.st.s[buf] + k0 * kStride;
+#pragma unroll
+                    for (int k = 0; k < kKahan; ++k) {
+                        const float4 q = Q[k * kStride + kTileY / 4];
+                        float d = __fadd_rn(rxh, q.z);
+                        if (LO) d = __fadd_rn(d, rxl);
+                        const float d2 = __fmul_rn(d, d);
+                        const float2 dx = f2(d, d), dx2 = f2(d2, d2), m2 = f2(q.x, q.y);
+                        float4 row[NP / 2];
+#pragma unroll
+                        for (int h = 0; h < NP / 2; ++h) row[h] = Q[k * kStride + tg * (NP / 2) + h];
+#pragma unroll
+                        for (int p = 0; p < NP; ++p) {
+                            const float2 dy = p % 2 ? f2(row[p / 2].z, row[p / 2].w) : f2(row[p / 2].x, row[p / 2].y);
+                            const float2 r2 = __ffma2_rn(dy, dy, dx2);
+                            const float2 inv =
+                                NRP > 0 && p == 0 && k % 3 == 2 ? rcp_nr2(r2) : f2(rcp_approx(r2.x), rcp_approx(r2.y));
+                            const float2 f = __fmul2_rn(m2, inv);
+                            px[p] = __ffma2_rn(f, dx, px[p]);
+                            py[p] = __ffma2_rn(f, dy, py[p]);
+                        }
+                    }
 #pragma unroll
                     for (int p = 0; p < NP; ++p) {
                         kahan2(Sx[p], Cx[p], px[p]);
@@ -326,18 +380,18 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
                         px[p] = py[p] = f2(0.f, 0.f);
                     }
                 }
-            }
-        };
-        if (LOM == 2 && !NAIVE)
-            chunks(std::true_type{});
-        else if (LOM == 1 || NAIVE)
-            chunks(std::false_type{});
-        else if (lo)
-            chunks(std::true_type{});
-        else
-            chunks(std::false_type{});
-        if (s + 1 < nstage) stage_store(buf ^ 1);
-        __syncthreads();
+            };
+            if (LOM == 2)
+                chunks(std::true_type{});
+            else if (LOM == 1)
+                chunks(std::false_type{});
+            else if (lo)
+                chunks(std::true_type{});
+            else
+                chunks(std::false_type{});
+            if (s + 1 < nstage) stage_store(buf ^ 1);
+            __syncthreads();
+        }
     }
 
     if constexpr (GS == 1) {
@@ -374,8 +428,10 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
     }
 
     if constexpr (SPLIT > 1) {
+        static_assert(sizeof(sm) >= 2 * NP * kThreads * sizeof(float4), "the partials fit the stage memory");
         cg::cluster_group cl = cg::this_cluster();
         const unsigned rank = cl.block_rank();
+        float4 *part = reinterpret_cast<float4 *>(&sm);  // the stages are dead (the loop's last barrier)
         if (rank != 0) {
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
@@ -412,8 +468,8 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
             if (!NAIVE) {
                 const float sx = h ? Sx[p].y : Sx[p].x, sy = h ? Sy[p].y : Sy[p].x;
                 const float ccx = h ? Cx[p].y : Cx[p].x, ccy = h ? Cy[p].y : Cy[p].x;
-                const float dxr = rx.x, dyr = h ? ry[p].y : ry[p].x;
-                const float dxl = rxl.x, dyl = h ? ryl[p].y : ryl[p].x;
+                const float dxr = rxh, dyr = ts.ro[tg * 2 * NP + r];
+                const float dxl = rxl, dyl = ts.rl[tg * 2 * NP + r];
                 // A delta for this ray (small), the offsets' low parts included
                 const float lx = __fmaf_rn(a.lens.fa11, dxr, __fmaf_rn(a.lens.fa12, dyr,
                                            __fmaf_rn(a.lens.fa11, dxl, __fmul_rn(a.lens.fa12, dyl))));
@@ -427,8 +483,8 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
                 tl = __fadd_rn(tl, __fadd_rn(__fadd_rn(ts.tc[7], ccy), ly));
                 two_sum(th, tl, byh[r], byl[r]);
             } else {
-                const float thy = h ? ry[p].y : ry[p].x;
-                bxh[r] = __fsub_rn(rx.x, h ? px[p].y : px[p].x);
+                const float thy = (float)R.y0 + ((float)(j0 + tg * 2 * NP + r) + 0.5f) * (float)R.dy;
+                bxh[r] = __fsub_rn(rxh, h ? px[p].y : px[p].x);
                 byh[r] = __fsub_rn(thy, h ? py[p].y : py[p].x);
                 bxl[r] = 0.0f;
                 byl[r] = 0.0f;
