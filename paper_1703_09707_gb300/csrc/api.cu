@@ -99,12 +99,28 @@ AxisPair make_axis(double x0, double x1, int n)
     a.x0l = (float)(x0 - (double)a.x0h);
     a.sh = (float)s;
     a.sl = (float)(s - (double)a.sh);
-    a.sh2 = 2.0f * std::fabs(a.sh);
-    const double tq = 2.0 * std::fabs((double)a.x0l) * std::fabs((double)a.sh) + 0x1p-100;
-    a.tq = (float)tq;
-    if ((double)a.tq < tq) a.tq = std::nextafter(a.tq, INFINITY);
     a.n = n;
     return a;
+}
+
+// One axis' constants of the fast pixel rule (the bound is derived at fast_pixel).
+void make_fast(const AxisPair &a, double x0, double s, float &nx0, float &sc, float &c, float &thr, float &blmax)
+{
+    nx0 = -a.x0h;
+    sc = a.sh;
+    const double cd = -(x0 - (double)a.x0h) * s - 0.5;
+    c = (float)cd;
+    const double del = 0x1p-24 * 1.001 * (3.0 * a.n + 4.0 * std::fabs(cd) + 8.0);
+    const double t = 0.5 - del, bm = 0.25 / std::fabs((double)a.sh);
+    thr = (float)t;
+    if ((double)thr > t) thr = std::nextafter(thr, -INFINITY);
+    blmax = (float)bm;
+    if ((double)blmax > bm) blmax = std::nextafter(blmax, 0.0f);
+    // pixel numbers must stay within the magic number's range, and the map's origin
+    // within 2^21 pixels of 0, so that a normalised pair's low part is below a quarter
+    // pixel wherever its high part is near the map
+    if (!(t > 0.0) || a.n > (1 << 20) || !(std::fabs(x0 * s) <= 0x1p21) || !std::isfinite(blmax) || !(blmax > 0.0f))
+        thr = -1.0f;
 }
 
 int read_stats(unsigned long long *d_stats, uint64_t total, mlens_stats *st, cudaStream_t s)
@@ -268,6 +284,9 @@ BinGrid make_bin_grid(const mlens_grid &g)
     BinGrid b;
     b.ax = make_axis(g.x0, g.x1, g.nx);
     b.ay = make_axis(g.y0, g.y1, g.ny);
+    FastBin &f = b.fast;
+    make_fast(b.ax, g.x0, (double)g.nx / (g.x1 - g.x0), f.nx0.x, f.s.x, f.c.x, f.thr.x, f.blmax.x);
+    make_fast(b.ay, g.y0, (double)g.ny / (g.y1 - g.y0), f.nx0.y, f.s.y, f.c.y, f.thr.y, f.blmax.y);
     b.x0 = g.x0;
     b.x1 = g.x1;
     b.y0 = g.y0;

@@ -1609,34 +1609,24 @@ __device__ __forceinline__ void learned_tile(const LearnedArgs &L, int bx, int b
     __syncthreads();
     hist_zero(sm.hist);
     if (tid == 0) {
-        ts.win[0] = pair_axis_rough(bxh[0], a.bin.ax) - kWin / 2;
-        ts.win[1] = pair_axis_rough(byh[0], a.bin.ay) - kWin / 2;
+        ts.win[0] = win_origin(pair_axis_rough(bxh[0], a.bin.ax), a.bin.nx);
+        ts.win[1] = win_origin(pair_axis_rough(byh[0], a.bin.ay), a.bin.ny);
     }
     __syncthreads();
-    WinHist W{sm.hist, ts.win[0], ts.win[1]};
-    unsigned nb = 0, no = 0, nn = 0;
+    const WinHist W = make_window(sm.hist, ts.win[0], ts.win[1], a.bin);
+    const int nrow = col_ok ? min(2 * NP, R.ny - (j0 + tg * 2 * NP)) : 0;  // this thread's rays in the grid
+    unsigned no = 0, nn = 0;
 #pragma unroll
     for (int r = 0; r < 2 * NP; ++r) {
-        const int jy = j0 + tg * 2 * NP + r;
-        uint32_t key = kNoKey;
-        if (col_ok && jy < R.ny) {
-            int gpx = 0, gpy = 0;
-            const int pix = pair_pixel(bxh[r], byh[r], bxl[r], byl[r], a.bin, gpx, gpy);
-            if (pix >= 0) {
-                ++nb;
-                key = hist_key(pix, gpx, gpy, W, a.bin);
-            } else if (pix == -1) {
-                ++no;
-            } else {
-                ++nn;
-            }
+        if (r < nrow) {
+            bin_pair<true>(bxh[r], byh[r], bxl[r], byl[r], a.bin, W, a.counts, no, nn);
             if (a.beta_out) {
                 float4 *bo = reinterpret_cast<float4 *>(a.beta_out);
-                bo[(int64_t)jy * R.nx + ix] = make_float4(bxh[r], byh[r], bxl[r], byl[r]);
+                bo[(int64_t)(j0 + tg * 2 * NP + r) * R.nx + ix] = make_float4(bxh[r], byh[r], bxl[r], byl[r]);
             }
         }
-        hist_add_warp(key, W, a.counts);
     }
+    const unsigned nb = (unsigned)max(nrow, 0) - no - nn;
     __syncthreads();
     hist_flush(W, a.bin, a.counts);
     stats_add_block(nb, no, nn, ts.sred, a.stats);

@@ -21,12 +21,21 @@ constexpr float kPadCoord = 1.0e15f;
 // s = n / (x1 - x0) = sh + sl, each split from its double value.
 struct AxisPair {
     float x0h, x0l, sh, sl;
-    float sh2;  // 2 |sh|
-    float tq;   // 2 |x0l| |sh| + 2^-100, rounded up: the constant part of the quick test's bound
     int n;
 };
 
+// Constants of the fast pixel rule (fast_pixel in mlens_dev.cuh), the x and y axes in
+// the two lanes; made by make_bin_grid.
+struct FastBin {
+    float2 nx0;    // -x0h
+    float2 s;      // sh
+    float2 c;      // -x0l s - 1/2
+    float2 thr;    // decided when |u - nearest integer| <= thr: 1/2 less the rule's error bound; -1: never
+    float2 blmax;  // the rule holds for |bl| <= blmax (a quarter pixel)
+};
+
 struct BinGrid {
+    FastBin fast;
     AxisPair ax, ay;
     double x0, x1, y0, y1;  // the double box, for the FP64 rule
     int nx, ny;
