@@ -271,8 +271,8 @@ int mlens_bin_grid(const void *beta_dev, const mlens_grid *rays, const mlens_gri
  *              CUDA graph); with NULL the library allocates the workspace (4
  *              bytes per pixel for the Gaussian, 8 for the disk), frees it
  *              before returning, and so synchronises `stream`.
- * The weights / half-widths are computed on the device from the definition
- * above (FP64, no contraction).  Errors: MLENS_ERR_ARG, MLENS_ERR_NOMEM,
+ * The weights / half-widths are computed from the definition above in FP64
+ * without contraction.  Errors: MLENS_ERR_ARG, MLENS_ERR_NOMEM,
  * MLENS_ERR_CUDA.
  */
 int mlens_convolve(const uint32_t *counts_dev, const mlens_grid *src, int32_t profile, double size, double scale,

@@ -6,13 +6,15 @@
 //   out[j][i] = scale * sum_{(di,dj) in K} w(di,dj) counts[j+dj][i+di],
 //   counts = 0 outside the map, weights normalised to sum 1 over K.
 //
-// Gaussian profile: separable, so two HBM-bound passes over the map -- rows
+// Gaussian profile: separable, so two passes over the map -- rows
 // (uint32 counts -> FP32) and columns (FP32 -> FP32 x scale) -- each staging a
 // tile plus its halo in shared memory and taking every tap from there.
 // Uniform disk: each row of the disk's support is one contiguous run of pixels,
-// so with per-row inclusive prefix sums P (int64, exact) an output is
+// so with per-row inclusive prefix sums P an output is
 // sum over the support's rows of P[row][i+h] - P[row][i-h-1]: O(rows) work per
-// pixel, exact integer sums, then (float)(sum * (scale / |K|)) in FP64.
+// pixel, exact integer sums, then (float)(sum * (scale / |K|)) as FP64 rounds it.
+// One kernel with the prefixes in shared memory where a tile fits, else prefixes in
+// int64 in global memory.
 // Light curve: bilinear interpolation between pixel centres along a straight
 // source track, in FP64 with explicit round-to-nearest operations.
 #include <cuda_runtime.h>
@@ -28,121 +30,174 @@ namespace mlens {
 namespace {
 
 constexpr int kThr = 256;
-constexpr int kRowOut = 1024;   // row pass: outputs per CTA
 constexpr int kColX = 64;       // column pass: tile columns
 constexpr int kColY = 128;      // column pass: tile rows
 constexpr int kMaxTaps = 256;   // Gaussian half-width limit (pixels)
 constexpr int kMaxDiskRows = 4096;
+constexpr size_t kDiskTileSmem3 = 74 * 1024;   // three CTAs per SM
+constexpr size_t kDiskTileSmem1 = 220 * 1024;  // one
+
+// Asynchronous global -> shared copy of N = 4 or 16 bytes (cp.async: no register round
+// trip, so all of a thread's copies are in flight at once); ok = false writes zeros
+// and reads nothing.
+template <int N>
+__device__ __forceinline__ void cp_async(void *smem, const void *gmem, bool ok)
+{
+    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;\n" ::"r"(s), "l"(gmem), "n"(N), "r"(ok ? N : 0) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
 
 __host__ __device__ constexpr int taps_padded(int K) { return (2 * K + 1 + 3) / 4 * 4; }
 
 __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
-// Row pass.  A CTA takes kRowOut outputs of two adjacent rows; thread t computes
-// the four consecutive outputs 4t .. 4t+3 of both rows, the rows packed into the
-// two lanes of f32x2 registers (FFMA2), with a sliding window stepped four taps
-// at a time: per four taps two float4 loads of duplicated weights (broadcast),
-// four float2 input loads and sixteen FFMA2 = 32 multiply-adds.  Each output
-// takes its taps in the same order as a scalar loop would: the packing changes
-// no result.  The weights are zero-padded to a multiple of four (adding exact
-// zeros).  The staged inputs are stored de-interleaved by index mod 4 (plane
-// e % 4, slot e / 4) so that the lanes' loads of element 4t + k are consecutive.
-__global__ void __launch_bounds__(kThr) k_gauss_rows(const uint32_t *__restrict__ in, int nx, int ny,
-                                                     const float *__restrict__ w, int K, float *__restrict__ out)
+// The normalised 1-D weights, zero-padded to a multiple of four (adding exact zeros),
+// passed by value with the launch: every thread of the grid takes the same weight at
+// the same time, so they come from the constant bank.  From shared memory, duplicated
+// for the packed arithmetic, they took as much of its bandwidth as the pixels did and
+// bound both passes.
+struct GaussTaps {
+    float w[taps_padded(kMaxTaps)];
+};
+
+// acc[q] += sum_t w_t x[q + t] for N outputs and one step of four taps, every output's taps
+// in ascending order.  Tap by tap over the outputs, so that consecutive packed
+// operations share the weight operand (three distinct operand pairs cost a third
+// cycle).
+template <int N>
+__device__ __forceinline__ void gauss_step(float2 (&acc)[N], const float2 (&x)[N + 3], const float *w)
 {
-    extern __shared__ float4 sm4[];
-    const int Kp = taps_padded(K);
-    float2 *ws = reinterpret_cast<float2 *>(sm4);  // Kp weights, each duplicated (w, w)
-    const int E = kRowOut + Kp + 3;                // staged inputs per row
-    const int P = E / 4 + 1;
-    float2 *xs = ws + Kp;                          // 4 planes of P (row j, row j + 1) pairs
-    const int tid = threadIdx.x;
-    for (int k = tid; k < Kp; k += kThr) {
-        const float v = k <= 2 * K ? w[k] : 0.0f;
-        ws[k] = make_float2(v, v);
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+        const float2 wt = make_float2(w[t], w[t]);
+#pragma unroll
+        for (int q = 0; q < N; ++q) acc[q] = ffma2(wt, x[q + t], acc[q]);
     }
-    const int i0 = blockIdx.x * kRowOut;
-    const int o = 4 * tid;  // this thread's first output within the tile
-    for (int64_t j = 2 * (int64_t)blockIdx.y; j < ny; j += 2 * (int64_t)gridDim.y) {
-        const bool two = j + 1 < ny;
+}
+
+// Row pass.  TX threads take 8 TX consecutive outputs of two adjacent rows, thread t
+// outputs 8t .. 8t+7 of both, the rows packed into the lanes of f32x2 registers, with
+// a sliding window of 11 inputs stepped four taps at a time: four 8-byte shared-memory
+// loads per 32 packed multiply-adds.  A CTA holds kThr / TX row pairs.  The staged
+// inputs are de-interleaved by index mod 8 (plane e % 8, slot e / 8) so that the lanes'
+// loads of element 8t + k are consecutive.  TX follows the map's width (run_convolution):
+// 1024 outputs per row pair need the least halo, narrower maps would leave threads
+// without outputs.
+// Bound by the FP32 pipe and the staging's latency: 83 taps over 4096^2 pixels 83 ->
+// 71 us (the multiply-adds alone take 35 us); the whole call 182 -> 131 us, 300 x 2000
+// pixels and 97 taps 37 -> 21 us.
+template <int TX>
+__global__ void __launch_bounds__(kThr) k_gauss_rows(const uint32_t *__restrict__ in, int nx, int ny,
+                                                     const __grid_constant__ GaussTaps W, int K,
+                                                     float *__restrict__ out)
+{
+    extern __shared__ float2 sm2[];
+    const int Kp = taps_padded(K);
+    const int E = 8 * TX + Kp + 7;  // staged inputs per row
+    const int P = E / 8 + 1;
+    const int t = threadIdx.x % TX, g = threadIdx.x / TX;
+    float2 *xs = sm2 + g * 8 * P;
+    const int i0 = blockIdx.x * 8 * TX;
+    constexpr int kPairs = kThr / TX;
+    for (int64_t jb = 2 * kPairs * (int64_t)blockIdx.y; jb < ny; jb += 2 * kPairs * (int64_t)gridDim.y) {
+        const int64_t j = jb + 2 * g;
+        const bool one = j < ny, two = j + 1 < ny;
         const uint32_t *row0 = in + j * nx, *row1 = row0 + nx;
         __syncthreads();  // previous rows' taps are done
-        for (int e = tid; e < E; e += kThr) {
-            const int i = i0 - K + e;
-            const bool inside = i >= 0 && i < nx;
-            xs[(e & 3) * P + (e >> 2)] =
-                make_float2(inside ? (float)row0[i] : 0.0f, inside && two ? (float)row1[i] : 0.0f);
+        constexpr int kB = 5;  // elements of each row in flight per thread
+        for (int e0 = t; e0 < E; e0 += kB * TX) {
+            uint32_t v0[kB], v1[kB];
+#pragma unroll
+            for (int q = 0; q < kB; ++q) {
+                const int e = e0 + q * TX, i = i0 - K + e;
+                const bool inside = e < E && i >= 0 && i < nx;
+                v0[q] = inside && one ? row0[i] : 0u;
+                v1[q] = inside && two ? row1[i] : 0u;
+            }
+#pragma unroll
+            for (int q = 0; q < kB; ++q) {
+                const int e = e0 + q * TX;
+                if (e < E) xs[(e & 7) * P + (e >> 3)] = make_float2((float)v0[q], (float)v1[q]);
+            }
         }
         __syncthreads();
-        if (i0 + o < nx) {
-            // element 4t + 4m + d sits in plane d & 3, slot t + m + (d >> 2)
-            const float2 *b = xs + tid;
-            const float4 *wq = sm4;  // (w_2n, w_2n, w_2n+1, w_2n+1)
-            float2 a0 = make_float2(0.f, 0.f), a1 = a0, a2 = a0, a3 = a0;
-            float2 x0 = b[0], x1 = b[P], x2 = b[2 * P];
-            // (unrolled so that the next steps' loads issue ahead of this step's FFMA2s)
-#pragma unroll 8
-            for (int m = 0; m < Kp / 4; ++m) {
-                const float4 qa = wq[2 * m], qb = wq[2 * m + 1];
-                const float2 w0 = make_float2(qa.x, qa.y), w1 = make_float2(qa.z, qa.w);
-                const float2 w2 = make_float2(qb.x, qb.y), w3 = make_float2(qb.z, qb.w);
-                const float2 x3 = b[3 * P + m], x4 = b[m + 1], x5 = b[P + m + 1], x6 = b[2 * P + m + 1];
-                a0 = ffma2(w0, x0, a0); a1 = ffma2(w0, x1, a1); a2 = ffma2(w0, x2, a2); a3 = ffma2(w0, x3, a3);
-                a0 = ffma2(w1, x1, a0); a1 = ffma2(w1, x2, a1); a2 = ffma2(w1, x3, a2); a3 = ffma2(w1, x4, a3);
-                a0 = ffma2(w2, x2, a0); a1 = ffma2(w2, x3, a1); a2 = ffma2(w2, x4, a2); a3 = ffma2(w2, x5, a3);
-                a0 = ffma2(w3, x3, a0); a1 = ffma2(w3, x4, a1); a2 = ffma2(w3, x5, a2); a3 = ffma2(w3, x6, a3);
-                x0 = x4;
-                x1 = x5;
-                x2 = x6;
+        const int o = i0 + 8 * t;  // this thread's first output
+        float2 acc[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc[q] = make_float2(0.f, 0.f);
+        if (o < nx && one) {
+            const float2 *b = xs + t;  // element 8t + n: plane n % 8, slot t + n / 8
+            float2 x[11];
+#pragma unroll
+            for (int q = 0; q < 7; ++q) x[q] = b[q * P];
+            auto step = [&](int m, int half) {  // taps m .. m + 3, m = 4 half mod 8
+#pragma unroll
+                for (int q = 7; q < 11; ++q) {
+                    const int n = q + 4 * half;  // plane and slot of element m + q, relative to m's eight
+                    x[q] = b[(n & 7) * P + (m >> 3) + (n >> 3)];
+                }
+                gauss_step<8>(acc, x, W.w + m);
+#pragma unroll
+                for (int q = 0; q < 7; ++q) x[q] = x[q + 4];
+            };
+            int m = 0;
+#pragma unroll 2
+            for (; m + 8 <= Kp; m += 8) {
+                step(m, 0);
+                step(m + 4, 1);
             }
-            const int n = min(4, nx - (i0 + o));
-            float *orow = out + j * nx + i0 + o;
-            orow[0] = a0.x;
-            if (n > 1) orow[1] = a1.x;
-            if (n > 2) orow[2] = a2.x;
-            if (n > 3) orow[3] = a3.x;
-            if (two) {
-                orow += nx;
-                orow[0] = a0.y;
-                if (n > 1) orow[1] = a1.y;
-                if (n > 2) orow[2] = a2.y;
-                if (n > 3) orow[3] = a3.y;
-            }
+            if (m < Kp) step(m, 0);
         }
+        // outputs through the planes, so that the lanes store consecutive pixels (a
+        // thread's own eight would touch a sector per lane and store)
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 8; ++q) xs[q * P + t] = acc[q];
+        __syncthreads();
+        if (one)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int e = q * TX + t, i = i0 + e;
+                if (i < nx) {
+                    const float2 v = xs[(e & 7) * P + (e >> 3)];
+                    out[j * nx + i] = v.x;
+                    if (two) out[(j + 1) * nx + i] = v.y;
+                }
+            }
     }
 }
 
 // Column pass.  A CTA stages kColY + Kp + 3 rows of 64 columns; thread (p, g)
 // computes rows 16g .. 16g+15 of the adjacent columns 2p and 2p + 1 (packed into
-// f32x2 lanes) in blocks of eight consecutive rows, with the same four-taps-at-a-
-// time window (the lanes of a warp read 32 consecutive column pairs of one staged
-// row).  As in the row pass, every output's taps keep their order.
+// f32x2 lanes) in blocks of eight consecutive rows, with the same window (the lanes of a
+// warp read 32 consecutive column pairs of one staged row).  As in the row pass, every
+// output's taps keep their order.  VEC: rows of 16-byte-aligned chunks, staged 16 bytes at
+// a time.  Bound by the FP32 pipe (74 % busy): 80 -> 57 us at the size above.
+template <bool VEC>
 __global__ void __launch_bounds__(kThr) k_gauss_cols(const float *__restrict__ in, int nx, int ny,
-                                                     const float *__restrict__ w, int K, float scale,
+                                                     const __grid_constant__ GaussTaps W, int K, float scale,
                                                      float *__restrict__ out)
 {
-    extern __shared__ float4 sm4[];
+    extern __shared__ __align__(16) float tile[];  // (kColY + Kp + 3) rows x kColX columns
     const int Kp = taps_padded(K);
-    float2 *ws = reinterpret_cast<float2 *>(sm4);        // Kp weights, each duplicated (w, w)
-    float *tile = reinterpret_cast<float *>(ws + Kp);    // (kColY + Kp + 3) rows x kColX columns
     const int tid = threadIdx.x;
-    for (int k = tid; k < Kp; k += kThr) {
-        const float v = k <= 2 * K ? w[k] : 0.0f;
-        ws[k] = make_float2(v, v);
-    }
-    const int lc = tid % kColX, lg = tid / kColX;        // staging: column, row group
-    const int cp = tid % (kColX / 2), g = tid / (kColX / 2);  // compute: column pair, group of kColY / 8 rows
-    const int il = blockIdx.x * kColX + lc;
-    const int i = blockIdx.x * kColX + 2 * cp;           // first column of this thread's pair
+    const int cp = tid % (kColX / 2), g = tid / (kColX / 2);  // column pair, group of kColY / 8 rows
+    const int ib = blockIdx.x * kColX;
+    const int i = ib + 2 * cp;                                // first column of this thread's pair
     const int rows = kColY + Kp + 3;
     const int tiles_y = (ny + kColY - 1) / kColY;
     for (int ty = blockIdx.y; ty < tiles_y; ty += gridDim.y) {
         const int64_t j0 = (int64_t)ty * kColY;
         __syncthreads();
-        for (int r = lg; r < rows; r += kThr / kColX) {
+        constexpr int kChunk = VEC ? 4 : 1, kPerRow = kColX / kChunk;
+        const int lc = kChunk * (tid % kPerRow);
+        for (int r = tid / kPerRow; r < rows; r += kThr / kPerRow) {
             const int64_t j = j0 - K + r;
-            tile[r * kColX + lc] = (il < nx && j >= 0 && j < ny) ? in[j * nx + il] : 0.0f;
+            const bool ok = ib + lc < nx && j >= 0 && j < ny;
+            cp_async<4 * kChunk>(tile + r * kColX + lc, ok ? in + j * nx + ib + lc : in, ok);
         }
+        cp_async_wait_all();
         __syncthreads();
         if (i >= nx) continue;
         const bool two = i + 1 < nx;
@@ -150,25 +205,16 @@ __global__ void __launch_bounds__(kThr) k_gauss_cols(const float *__restrict__ i
             if (j0 + r >= ny) break;
             const float2 *T = reinterpret_cast<const float2 *>(tile + r * kColX + 2 * cp);
             constexpr int S = kColX / 2;  // float2 per staged row
-            float2 a[8], x[11];
+            float2 acc[8], x[11];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) a[q] = make_float2(0.f, 0.f);
+            for (int q = 0; q < 8; ++q) acc[q] = make_float2(0.f, 0.f);
 #pragma unroll
             for (int q = 0; q < 7; ++q) x[q] = T[q * S];
 #pragma unroll 4
             for (int k = 0; k < Kp; k += 4) {
-                const float4 qa = sm4[k >> 1], qb = sm4[(k >> 1) + 1];
-                const float2 w0 = make_float2(qa.x, qa.y), w1 = make_float2(qa.z, qa.w);
-                const float2 w2 = make_float2(qb.x, qb.y), w3 = make_float2(qb.z, qb.w);
 #pragma unroll
-                for (int q = 0; q < 4; ++q) x[7 + q] = T[(k + 7 + q) * S];
-#pragma unroll
-                for (int q = 0; q < 8; ++q) {
-                    a[q] = ffma2(w0, x[q], a[q]);
-                    a[q] = ffma2(w1, x[q + 1], a[q]);
-                    a[q] = ffma2(w2, x[q + 2], a[q]);
-                    a[q] = ffma2(w3, x[q + 3], a[q]);
-                }
+                for (int q = 7; q < 11; ++q) x[q] = T[(k + q) * S];
+                gauss_step<8>(acc, x, W.w + k);
 #pragma unroll
                 for (int q = 0; q < 7; ++q) x[q] = x[q + 4];
             }
@@ -176,8 +222,8 @@ __global__ void __launch_bounds__(kThr) k_gauss_cols(const float *__restrict__ i
             for (int q = 0; q < 8; ++q)
                 if (j0 + r + q < ny) {
                     float *dst = out + (j0 + r + q) * nx + i;
-                    dst[0] = __fmul_rn(a[q].x, scale);
-                    if (two) dst[1] = __fmul_rn(a[q].y, scale);
+                    dst[0] = __fmul_rn(acc[q].x, scale);
+                    if (two) dst[1] = __fmul_rn(acc[q].y, scale);
                 }
         }
     }
@@ -269,119 +315,207 @@ __global__ void __launch_bounds__(kThr) k_disk(const int64_t *__restrict__ P, in
     }
 }
 
-// The same sums for disks of moderate size, with the prefix sums a tile needs staged
-// in shared memory once: a CTA takes kDiskTX x kDiskTY outputs and loads rows
-// j0 - H .. j0 + kDiskTY - 1 + H, columns i0 - W - 1 .. i0 + kDiskTX - 1 + W of P
-// (W: the largest half-width), with 0 above and below the map and left of it and
-// P[row][nx - 1] right of it -- exactly the values k_disk's clamps produce, so the
-// integer sums, and the outputs, are identical.  The 2 (2H + 1) loads per output
-// then come from shared memory instead of L2.  Thread (c, g) computes column c of
-// rows 8 g .. 8 g + 7 of the tile.
-constexpr int kDiskTX = 64, kDiskTY = 32;
+// The same sums for disks of moderate size, in one kernel straight from the counts: a
+// CTA takes TX x TY outputs, stages the counts they need (TY + 2H rows, TX + 2W + 1
+// columns; zero outside the map) and turns each staged row into its prefix sums in
+// place.  An output is the sum over the support's rows of two prefix values' difference;
+// thread (c, g) computes column c, eight rows at a time, taking the support's rows in
+// groups of equal half-width: m such rows need m + 7 run sums for the eight outputs, not 8 m.
+// The row stride S is a template parameter, so that the rows' loads have immediate
+// addresses; S = 4 x odd, four segments of S / 4 words: the scan's 8 rows x 4 segments
+// per warp fall on 32 different banks.
+// Sums are exact in 32 bits, modulo 2^32 in the prefixes, while the largest staged count
+// times |K| is below 2^32 (`limit`; 3.2e6 rays in a pixel for 1317 pixels).  A tile with
+// larger counts takes its sums from the counts' low and high halves in two passes per eight
+// rows, in 64 bits.
+// Bound by shared-memory loads, 59 of 4 bytes per output at R = 20 pixels: 4096^2 pixels in
+// 164 us, 373 us with int64 prefixes made by a kernel of their own and staged with their
+// halo (8 bytes a load, and three FP64 operations per output); R = 45 1959 -> 456 us.
+constexpr int kMaxGroups = 256;  // runs of support rows of one half-width that a plan carries
+struct DiskGroups {
+    int n;
+    uint16_t half[kMaxGroups], rows[kMaxGroups];
+};
 
-// 8-byte asynchronous global -> shared copy (Ampere-style cp.async: no register round
-// trip, so all of a thread's copies are in flight at once); n = 0 writes zeros and
-// reads nothing.
-__device__ __forceinline__ void cp_async8(void *smem, const void *gmem, int n)
+// The groups cut into blocks of 8, 4, 2 and 1 rows (integer sums take any order), each the
+// stage offsets of its first row's upper and lower prefix value; passed by value with
+// the launch and read from the constant bank.
+constexpr int kMaxBlocks = 384;
+struct DiskBlocks {
+    int n8, n4, n2, n1;  // ends of the blocks of each kind
+    int2 at[kMaxBlocks];
+};
+static_assert(sizeof(DiskBlocks) <= 3584, "fits the launch's parameters");
+
+// Columns of the support a tile of TX outputs and row stride S (words) has room for.
+constexpr int disk_tile_w(int TX, int S) { return (S - TX - 1) / 2; }
+
+// (float)((double)s * f), each operation rounded to nearest, without the FP64 pipe (two
+// conversions and a product cost more there than the sum itself).  With f = fh + fl + O(2^-48)
+// and s = sh + sl exact, p + t is s f to 2^-44 relative; r = fl(p + t) is the double
+// product's rounding to float whenever p + t (1 +- 2^-40 |p|) round to the same float, which
+// then holds of the double between them.  `fast` = |f| within 2^+-60.
+__device__ __noinline__ float scale_sum_fp64(uint32_t s, double f)  // out of line: never evaluated speculatively
 {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;\n" ::"r"(s), "l"(gmem), "r"(n) : "memory");
+    return __double2float_rn(__dmul_rn((double)s, f));
 }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;\n" ::: "memory"); }
-constexpr size_t kDiskTileMaxSmem = 100 * 1024;  // above this the plain kernel runs
-
-__host__ __device__ constexpr size_t disk_tile_smem(int H, int W)
+__device__ __forceinline__ float scale_sum(uint32_t s, double f, float fh, float fl, bool fast)
 {
-    return ((size_t)kDiskTY + 2 * (size_t)H) * ((size_t)kDiskTX + 2 * (size_t)W + 1) * sizeof(int64_t) +
-           (2 * (size_t)H + 1) * sizeof(int);  // size_t throughout: W can be as large as nx
+    const float sh = __uint2float_rn(s);
+    const float sl = (float)(int)(s - (sh >= 4294967296.0f ? 0u : (uint32_t)sh));
+    const float p = __fmul_rn(sh, fh);
+    const float e = __fmaf_rn(sh, fh, -p);
+    const float t = __fmaf_rn(sh, fl, __fmaf_rn(sl, fh, e));
+    const float z = __fmul_rn(fabsf(p), 0x1p-40f);
+    const float up = __fadd_rn(p, __fadd_rn(t, z)), dn = __fadd_rn(p, __fsub_rn(t, z));
+    if (s == 0u && fast) return p;  // the zero's sign is f's
+    if (fast && up == dn) return up;
+    return scale_sum_fp64(s, f);
 }
 
-__global__ void __launch_bounds__(kThr) k_disk_tile(const int64_t *__restrict__ P, int nx, int ny,
-                                                    const int *__restrict__ half, int H, int W, double f,
-                                                    float *__restrict__ out)
+template <int TX, int TY, int S>
+__global__ void __launch_bounds__(kThr) k_disk_tile(const uint32_t *__restrict__ in, int nx, int ny,
+                                                    const __grid_constant__ DiskBlocks B, int H, uint32_t limit,
+                                                    double f, float fh, float fl, bool fast, float *__restrict__ out)
 {
-    extern __shared__ __align__(16) unsigned char dsm[];
-    const int rows = kDiskTY + 2 * H, cols = kDiskTX + 2 * W + 1;
-    int64_t *T = reinterpret_cast<int64_t *>(dsm);
-    int *hs = reinterpret_cast<int *>(T + (size_t)rows * cols);
-    const int tid = threadIdx.x, c = tid % kDiskTX, g = tid / kDiskTX;
-    const int i0 = blockIdx.x * kDiskTX;
-    for (int k = tid; k <= 2 * H; k += kThr) hs[k] = min(half[k], W);  // half[k] <= W: a guard only
-    const int64_t tiles_y = ((int64_t)ny + kDiskTY - 1) / kDiskTY;
+    extern __shared__ __align__(16) uint32_t T[];
+    constexpr int kGroup = kThr / TX, kRows = 8, kPer = TY / kGroup;  // output rows per thread, kRows at a time
+    static_assert(kThr % TX == 0 && kPer % kRows == 0, "whole batches");
+    static_assert(S % 8 == 4, "conflict-free scan");
+    constexpr int W = disk_tile_w(TX, S);  // the staged columns start at i0 - W - 1
+    const int rows = TY + 2 * H;
+    const int tid = threadIdx.x, c = tid % TX, g = tid / TX;
+    const int i0 = blockIdx.x * TX, i = i0 + c;
+    const int64_t tiles_y = ((int64_t)ny + TY - 1) / TY;
     for (int64_t by = blockIdx.y; by < tiles_y; by += gridDim.y) {
-        const int64_t j0 = by * kDiskTY, jbase = j0 - H;
-        const int64_t cbase = (int64_t)i0 - W - 1;
-        __syncthreads();  // the previous tile's reads are done
-        for (int r = tid / 32; r < rows; r += kThr / 32) {  // a warp per row, its lanes along it
-            const int64_t jj = jbase + r;
-            const bool in = jj >= 0 && jj < ny;
-            for (int q = tid % 32; q < cols; q += 32) {
-                const int64_t col = cbase + q;
-                const bool ok = in && col >= 0;
-                cp_async8(&T[r * cols + q], ok ? P + jj * nx + (col < nx ? col : nx - 1) : P, ok ? 8 : 0);
+        const int64_t j0 = by * TY;
+        // stage the counts
+        auto stage = [&]() {
+            __syncthreads();  // the previous reads are done
+            for (int r = tid / 32; r < rows; r += kThr / 32) {  // a warp per row, its lanes along it
+                const int64_t jj = j0 - H + r;
+                const bool in_y = jj >= 0 && jj < ny;
+                const uint32_t *row = in + jj * nx;
+                for (int q = tid % 32; q < S; q += 32) {
+                    const int64_t col = (int64_t)i0 - W - 1 + q;
+                    const bool ok = in_y && col >= 0 && col < nx;
+                    cp_async<4>(&T[r * S + q], ok ? row + col : in, ok);
+                }
             }
-        }
-        cp_async_wait_all();
-        __syncthreads();
-        const int i = i0 + c;
-        if (i < nx) {
-            constexpr int kRows = kDiskTY / 4;  // output rows per thread
-            const int rt0 = g * kRows;          // the thread's first row within the tile
-            int64_t sum[kRows];
+            cp_async_wait_all();
+            __syncthreads();
+        };
+        // rows to prefix sums of (count >> shift) & mask, four lanes per row; returns the largest count seen
+        auto scan = [&](int shift, uint32_t mask) {
+            uint32_t top = 0;
+            for (int base = 0; base < rows; base += kThr / 4) {
+                const int r = base + tid / 4;
+                uint32_t *p = T + r * S + (tid & 3) * (S / 4);
+                uint32_t sum = 0;
+                if (r < rows) {
+#pragma unroll 8
+                    for (int k = 0; k < S / 4; ++k) {
+                        const uint32_t v = p[k];
+                        top = max(top, v);
+                        sum += (v >> shift) & mask;
+                    }
+                }
+                uint32_t inc = sum;  // inclusive over the row's four lanes
+#pragma unroll
+                for (int d = 1; d < 4; d <<= 1) {
+                    const uint32_t o = __shfl_up_sync(0xffffffffu, inc, d, 4);
+                    if ((tid & 3) >= d) inc += o;
+                }
+                uint32_t run = inc - sum;
+                if (r < rows) {
+#pragma unroll 8
+                    for (int k = 0; k < S / 4; ++k) {
+                        run += (p[k] >> shift) & mask;
+                        p[k] = run;
+                    }
+                }
+            }
+            return top;
+        };
+        // sums of the batch of eight rows from output row rt on
+        auto sums = [&](int rt, uint32_t (&sum)[kRows]) {
+            // row rt + d of the stage is row j0 + rt - H + d of the map; tr[0] is the column of i
+            const uint32_t *tr = T + rt * S + c + W;
 #pragma unroll
             for (int k = 0; k < kRows; ++k) sum[k] = 0;
-            // T row rt0 + d is row j0 + rt0 - H + d of the map; tr[0] is the column of i - 1.
-            // rs[k]: the run sum of output k at support row d.  Where the next support row
-            // has the same half-width (a warp-uniform test), output k's next run is output
-            // k + 1's current one, so the runs shift by one and only the last is loaded.
-            const int64_t *tr = T + (size_t)rt0 * cols + c + W;
-            int64_t rs[kRows];
-            int hprev = -1;
-            for (int d = 0; d <= 2 * H; ++d) {  // one half-width per support row, for all kRows outputs
-                const int h = hs[d];
-                if (h == hprev) {
+            int n = 0;
+            // run sum of row q of a block; a block of M rows adds run(k) + .. + run(k + M - 1) to output k
+            const uint32_t *hi, *lo;
+            auto run = [&](int q) { return hi[q * S] - lo[q * S]; };
+            for (; n < B.n8; ++n) {
+                hi = tr + B.at[n].x, lo = tr + B.at[n].y;
+                uint32_t r[kRows + 7];
 #pragma unroll
-                    for (int k = 0; k < kRows - 1; ++k) rs[k] = rs[k + 1];
-                    rs[kRows - 1] = tr[(kRows - 1) * cols + h + 1] - tr[(kRows - 1) * cols - h];
-                } else {
+                for (int q = 0; q < kRows + 7; ++q) r[q] = run(q);
 #pragma unroll
-                    for (int k = 0; k < kRows; ++k) rs[k] = tr[k * cols + h + 1] - tr[k * cols - h];
-                }
+                for (int q = 0; q < kRows + 6; ++q) r[q] += r[q + 1];
 #pragma unroll
-                for (int k = 0; k < kRows; ++k) sum[k] += rs[k];
-                hprev = h;
-                tr += cols;
+                for (int q = 0; q < kRows + 4; ++q) r[q] += r[q + 2];
+#pragma unroll
+                for (int k = 0; k < kRows; ++k) sum[k] += r[k] + r[k + 4];
             }
+            for (; n < B.n4; ++n) {
+                hi = tr + B.at[n].x, lo = tr + B.at[n].y;
+                uint32_t r[kRows + 3];
 #pragma unroll
-            for (int k = 0; k < kRows; ++k) {
-                const int64_t j = j0 + rt0 + k;
-                if (j < ny) out[j * nx + i] = __double2float_rn(__dmul_rn((double)sum[k], f));
+                for (int q = 0; q < kRows + 3; ++q) r[q] = run(q);
+#pragma unroll
+                for (int q = 0; q < kRows + 2; ++q) r[q] += r[q + 1];
+#pragma unroll
+                for (int k = 0; k < kRows; ++k) sum[k] += r[k] + r[k + 2];
+            }
+            for (; n < B.n2; ++n) {
+                hi = tr + B.at[n].x, lo = tr + B.at[n].y;
+                uint32_t r[kRows + 1];
+#pragma unroll
+                for (int q = 0; q < kRows + 1; ++q) r[q] = run(q);
+#pragma unroll
+                for (int k = 0; k < kRows; ++k) sum[k] += r[k] + r[k + 1];
+            }
+#pragma unroll 2
+            for (; n < B.n1; ++n) {
+                hi = tr + B.at[n].x, lo = tr + B.at[n].y;
+#pragma unroll
+                for (int k = 0; k < kRows; ++k) sum[k] += run(k);
+            }
+        };
+        stage();
+        const uint32_t top = scan(0, 0xffffffffu);
+        const bool large = __syncthreads_or(top > limit);
+        for (int b = 0; b < kPer; b += kRows) {
+            const int rt = g * kPer + b;
+            uint32_t sum[kRows];
+            if (!large) {
+                if (i < nx && j0 + rt < ny) {
+                    sums(rt, sum);
+#pragma unroll
+                    for (int k = 0; k < kRows; ++k)
+                        if (j0 + rt + k < ny) out[(j0 + rt + k) * nx + i] = scale_sum(sum[k], f, fh, fl, fast);
+                }
+            } else {
+                uint32_t hi[kRows];
+                stage();
+                scan(0, 0xffffu);
+                __syncthreads();
+                sums(rt, sum);
+                stage();
+                scan(16, 0xffffu);
+                __syncthreads();
+                sums(rt, hi);
+#pragma unroll
+                for (int k = 0; k < kRows; ++k)
+                    if (i < nx && j0 + rt + k < ny) {
+                        const int64_t s = (int64_t)sum[k] + ((int64_t)hi[k] << 16);
+                        out[(j0 + rt + k) * nx + i] = __double2float_rn(__dmul_rn((double)s, f));
+                    }
             }
         }
     }
-}
-
-// Normalised 1-D Gaussian weights exp(-((k-K) d)^2 / (2 sigma^2)) / sum, one CTA:
-// FP64 terms, a fixed-order tree sum, float results.
-__global__ void __launch_bounds__(kThr) k_gauss_weights(double sigma, double d, int K, float *__restrict__ w)
-{
-    __shared__ double e[2 * kMaxTaps + 1];
-    __shared__ double part[kThr];
-    const int tid = threadIdx.x;
-    double acc = 0.0;
-    for (int k = tid; k <= 2 * K; k += kThr) {
-        const double off = __dmul_rn((double)(k - K), d);
-        e[k] = exp(-__ddiv_rn(__dmul_rn(off, off), __dmul_rn(2.0, __dmul_rn(sigma, sigma))));
-        acc = __dadd_rn(acc, e[k]);
-    }
-    part[tid] = acc;
-    __syncthreads();
-    for (int h = kThr / 2; h > 0; h >>= 1) {
-        if (tid < h) part[tid] = __dadd_rn(part[tid], part[tid + h]);
-        __syncthreads();
-    }
-    const double sum = part[0];
-    for (int k = tid; k <= 2 * K; k += kThr) w[k] = __double2float_rn(__ddiv_rn(e[k], sum));
 }
 
 // Half-width of each row dj = q - H of the disk support: the largest h with
@@ -486,6 +620,7 @@ struct ConvPlan {
     int Hs = 0;            // disk: support rows |dj| <= Hs
     int Ws = 0;            // disk: the largest half-width, capped at nx
     int64_t count = 0;     // disk: |K|
+    DiskGroups groups{};   // disk: runs of support rows of one half-width (capped at nx); n = 0: too many
     size_t off_map = 0;    // workspace offset of the map-sized buffer
     size_t bytes = 0;      // workspace size
 };
@@ -526,11 +661,113 @@ int plan_convolution(const mlens_grid *src, int32_t profile, double size, ConvPl
         }
         pl->Hs = Hs;
         pl->count = count;
+        DiskGroups &G = pl->groups;
+        for (int dj = -Hs; dj <= Hs; ++dj) {
+            const int h = std::min(half_width(size, dx, dy, dj), nx);
+            if (G.n > 0 && G.half[G.n - 1] == h) {
+                ++G.rows[G.n - 1];
+            } else if (G.n < kMaxGroups && h <= 0xffff) {
+                G.half[G.n] = (uint16_t)h;
+                G.rows[G.n++] = 1;
+            } else {
+                G.n = 0;
+                break;
+            }
+        }
         pl->off_map = round256((size_t)(2 * Hs + 1) * sizeof(int));
         pl->bytes = pl->off_map + round256(npix * sizeof(int64_t));
         return MLENS_OK;
     }
     return lc_fail(MLENS_ERR_ARG, "unknown profile");
+}
+
+// Normalised 1-D Gaussian weights exp(-((k-K) d)^2 / (2 sigma^2)) / sum: FP64 terms
+// and sum, float results, zero-padded.
+GaussTaps gauss_taps(double sigma, double d, int K)
+{
+    GaussTaps t{};
+    std::vector<double> e((size_t)(2 * K + 1));
+    double sum = 0.0;
+    for (int k = 0; k <= 2 * K; ++k) {
+        const double off = (double)(k - K) * d;
+        e[(size_t)k] = std::exp(-(off * off) / (2.0 * (sigma * sigma)));
+        sum += e[(size_t)k];
+    }
+    for (int k = 0; k <= 2 * K; ++k) t.w[k] = (float)(e[(size_t)k] / sum);
+    return t;
+}
+
+template <int TX>
+cudaError_t launch_gauss_rows(const uint32_t *in, int nx, int ny, const GaussTaps &w, int K, float *out, cudaStream_t s)
+{
+    constexpr int kPairs = kThr / TX;
+    const size_t smem = (size_t)kPairs * 8 * ((8 * TX + taps_padded(K) + 7) / 8 + 1) * sizeof(float2);
+    const cudaError_t e = allow_dynamic_smem(k_gauss_rows<TX>, smem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)((nx + 8 * TX - 1) / (8 * TX)),
+                    (unsigned)std::min<int64_t>((ny + 2 * kPairs - 1) / (2 * kPairs), 65535));
+    k_gauss_rows<TX><<<grid, kThr, smem, s>>>(in, nx, ny, w, K, out);
+    return cudaGetLastError();
+}
+
+template <bool VEC>
+cudaError_t launch_gauss_cols(const float *in, int nx, int ny, const GaussTaps &w, int K, float scale, float *out,
+                              cudaStream_t s)
+{
+    const size_t smem = (size_t)(kColY + taps_padded(K) + 3) * kColX * sizeof(float);
+    const cudaError_t e = allow_dynamic_smem(k_gauss_cols<VEC>, smem);
+    if (e != cudaSuccess) return e;
+    const int64_t tiles_y = (ny + kColY - 1) / kColY;
+    const dim3 grid((unsigned)((nx + kColX - 1) / kColX), (unsigned)std::min<int64_t>(tiles_y, 65535));
+    k_gauss_cols<VEC><<<grid, kThr, smem, s>>>(in, nx, ny, w, K, scale, out);
+    return cudaGetLastError();
+}
+
+template <int TX, int TY, int S>
+cudaError_t launch_disk_tile(const uint32_t *in, int nx, int ny, const ConvPlan &pl, double f, float *out,
+                             cudaStream_t s)
+{
+    const size_t smem = (size_t)(TY + 2 * pl.Hs) * S * sizeof(uint32_t);
+    const cudaError_t e = allow_dynamic_smem(k_disk_tile<TX, TY, S>, smem);
+    if (e != cudaSuccess) return e;
+    DiskBlocks B{};
+    int n = 0, *end[4] = {&B.n8, &B.n4, &B.n2, &B.n1};
+    for (int kind = 0; kind < 4; ++kind) {
+        const int m = 8 >> kind;
+        for (int g = 0, row = 0; g < pl.groups.n; row += pl.groups.rows[g++]) {
+            const int h = pl.groups.half[g], all = pl.groups.rows[g];
+            // 8s first, then at most one block of each smaller kind, from the group's first row on
+            const int r0 = m == 8 ? 0 : all / (2 * m) * (2 * m), k = m == 8 ? all / 8 : all / m % 2;
+            for (int q = 0; q < k; ++q) {
+                if (n == kMaxBlocks) return cudaErrorInvalidValue;  // the plan has at most kMaxGroups groups: unreachable
+                const int r = (row + r0 + q * m) * S;
+                B.at[n++] = make_int2(r + h + 1, r - h);
+            }
+        }
+        *end[kind] = n;
+    }
+    const uint32_t limit = (uint32_t)(0xffffffffull / (uint64_t)pl.count);
+    const bool fast = std::fabs(f) > 0x1p-60 && std::fabs(f) < 0x1p60;
+    const float fh = (float)f, fl = (float)(f - (double)fh);
+    const dim3 grid((unsigned)((nx + TX - 1) / TX), (unsigned)std::min<int64_t>(((int64_t)ny + TY - 1) / TY, 65535));
+    k_disk_tile<TX, TY, S><<<grid, kThr, smem, s>>>(in, nx, ny, B, pl.Hs, limit, f, fh, fl, fast, out);
+    return cudaGetLastError();
+}
+
+// The disk in one kernel: 128 x 64 outputs (the least halo) where three CTAs fit an SM
+// and the tiles fill the SMs twice, else 64 x 32; the smallest row stride with room for
+// the support.  *done = false: no tile fits its shared memory.
+template <int TX, int TY, int S, int... More>
+cudaError_t disk_tile_of(const uint32_t *in, int nx, int ny, const ConvPlan &pl, double f, float *out, cudaStream_t s,
+                         size_t most, bool *done)
+{
+    if (pl.Ws <= disk_tile_w(TX, S)) {
+        if ((size_t)(TY + 2 * pl.Hs) * S * sizeof(uint32_t) > most) return cudaSuccess;
+        *done = true;
+        return launch_disk_tile<TX, TY, S>(in, nx, ny, pl, f, out, s);
+    }
+    if constexpr (sizeof...(More) > 0) return disk_tile_of<TX, TY, More...>(in, nx, ny, pl, f, out, s, most, done);
+    return cudaSuccess;
 }
 
 int run_convolution(const uint32_t *counts_dev, const mlens_grid *src, int32_t profile, double size, double scale,
@@ -540,50 +777,42 @@ int run_convolution(const uint32_t *counts_dev, const mlens_grid *src, int32_t p
     const double dx = (src->x1 - src->x0) / nx, dy = (src->y1 - src->y0) / ny;
     cudaError_t e;
     if (profile == MLENS_PROFILE_GAUSSIAN) {
-        float *wx = reinterpret_cast<float *>(work), *wy = wx + (2 * pl.Kx + 1);
         float *t = reinterpret_cast<float *>(work + pl.off_map);
-        k_gauss_weights<<<1, kThr, 0, s>>>(size, dx, pl.Kx, wx);
-        k_gauss_weights<<<1, kThr, 0, s>>>(size, dy, pl.Ky, wy);
-        if ((e = cudaGetLastError()) != cudaSuccess) return lc_cuda(e, "weights launch");
-        const int kpx = taps_padded(pl.Kx), kpy = taps_padded(pl.Ky);
-        const size_t sm_r = (size_t)(kpx + 4 * ((kRowOut + kpx + 3) / 4 + 1)) * sizeof(float2);
-        const size_t sm_c = (size_t)(2 * kpy + (kColY + kpy + 3) * kColX) * sizeof(float);
-        if ((e = cudaFuncSetAttribute(k_gauss_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_r)) !=
-                cudaSuccess ||
-            (e = cudaFuncSetAttribute(k_gauss_cols, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_c)) !=
-                cudaSuccess)
-            return lc_cuda(e, "cudaFuncSetAttribute");
-        const dim3 gr((unsigned)((nx + kRowOut - 1) / kRowOut), (unsigned)std::min<int64_t>((ny + 1) / 2, 65535));
-        k_gauss_rows<<<gr, kThr, sm_r, s>>>(counts_dev, nx, ny, wx, pl.Kx, t);
-        if ((e = cudaGetLastError()) != cudaSuccess) return lc_cuda(e, "row pass launch");
-        const int64_t tiles_y = (ny + kColY - 1) / kColY;
-        const dim3 gc((unsigned)((nx + kColX - 1) / kColX), (unsigned)std::min<int64_t>(tiles_y, 65535));
-        k_gauss_cols<<<gc, kThr, sm_c, s>>>(t, nx, ny, wy, pl.Ky, (float)scale, out_dev);
-        if ((e = cudaGetLastError()) != cudaSuccess) return lc_cuda(e, "column pass launch");
+        const GaussTaps wx = gauss_taps(size, dx, pl.Kx), wy = gauss_taps(size, dy, pl.Ky);
+        e = nx > 512 ? launch_gauss_rows<128>(counts_dev, nx, ny, wx, pl.Kx, t, s)
+                     : nx > 256 ? launch_gauss_rows<64>(counts_dev, nx, ny, wx, pl.Kx, t, s)
+                                : launch_gauss_rows<32>(counts_dev, nx, ny, wx, pl.Kx, t, s);
+        if (e != cudaSuccess) return lc_cuda(e, "row pass launch");
+        // the workspace is 256-byte aligned: rows of whole 16-byte chunks start on one
+        e = nx % 4 == 0 ? launch_gauss_cols<true>(t, nx, ny, wy, pl.Ky, (float)scale, out_dev, s)
+                        : launch_gauss_cols<false>(t, nx, ny, wy, pl.Ky, (float)scale, out_dev, s);
+        if (e != cudaSuccess) return lc_cuda(e, "column pass launch");
         return MLENS_OK;
     }
-    int *half = reinterpret_cast<int *>(work);
-    int64_t *P = reinterpret_cast<int64_t *>(work + pl.off_map);
     int dev = 0, nsm = 1;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return lc_cuda(e, "cudaGetDevice");
     if ((e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
         return lc_cuda(e, "cudaDeviceGetAttribute");
+    const double f = scale / (double)pl.count;
+    // One kernel from the counts wherever a tile fits (sums of 16-bit halves beyond 32
+    // bits need the 64-bit prefixes)
+    if (pl.groups.n > 0 && pl.count <= 65536) {
+        bool done = false;
+        if ((int64_t)((nx + 127) / 128) * ((ny + 63) / 64) >= 2 * (int64_t)nsm)
+            e = disk_tile_of<128, 64, 140, 172, 204>(counts_dev, nx, ny, pl, f, out_dev, s, kDiskTileSmem3, &done);
+        if (e == cudaSuccess && !done)
+            e = disk_tile_of<64, 32, 76, 108, 140, 172, 236, 300>(counts_dev, nx, ny, pl, f, out_dev, s, kDiskTileSmem1,
+                                                                  &done);
+        if (e != cudaSuccess) return lc_cuda(e, "disk launch");
+        if (done) return MLENS_OK;
+    }
+    int *half = reinterpret_cast<int *>(work);
+    int64_t *P = reinterpret_cast<int64_t *>(work + pl.off_map);
     k_disk_halves<<<(unsigned)((2 * pl.Hs + 1 + kThr - 1) / kThr), kThr, 0, s>>>(size, dx, dy, pl.Hs, nx, half);
     const unsigned gp = (unsigned)std::min<int64_t>(ny, (int64_t)nsm * 8);
     k_row_prefix<<<gp, kThr, 0, s>>>(counts_dev, nx, ny, P);
-    const size_t tsm = disk_tile_smem(pl.Hs, pl.Ws);
-    if (tsm <= kDiskTileMaxSmem) {
-        if ((e = cudaFuncSetAttribute(k_disk_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm)) !=
-            cudaSuccess)
-            return lc_cuda(e, "cudaFuncSetAttribute");
-        const dim3 gt((unsigned)((nx + kDiskTX - 1) / kDiskTX),
-                      (unsigned)std::min<int64_t>(((int64_t)ny + kDiskTY - 1) / kDiskTY, 65535));
-        k_disk_tile<<<gt, kThr, tsm, s>>>(P, nx, ny, half, pl.Hs, pl.Ws, scale / (double)pl.count, out_dev);
-    } else {
-        const dim3 gd((unsigned)((nx + kThr - 1) / kThr), (unsigned)std::min<int64_t>(ny, 65535));
-        k_disk<<<gd, kThr, (size_t)(2 * pl.Hs + 1) * sizeof(int), s>>>(P, nx, ny, half, pl.Hs,
-                                                                        scale / (double)pl.count, out_dev);
-    }
+    const dim3 gd((unsigned)((nx + kThr - 1) / kThr), (unsigned)std::min<int64_t>(ny, 65535));
+    k_disk<<<gd, kThr, (size_t)(2 * pl.Hs + 1) * sizeof(int), s>>>(P, nx, ny, half, pl.Hs, f, out_dev);
     if ((e = cudaGetLastError()) != cudaSuccess) return lc_cuda(e, "disk launches");
     return MLENS_OK;
 }
