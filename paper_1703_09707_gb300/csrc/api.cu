@@ -189,6 +189,7 @@ int shoot_impl(mlens_ctx *ctx, const mlens_grid *rays, const mlens_grid *src, ui
     if (row1 > row0) {
         const int ty0 = row0 / th, ty1 = (row1 + th - 1) / th;
         if (ctx->precision == MLENS_PREC_FP64) {
+            a.nstars = ctx->n;  // the padding adds exactly zero
             e = launch_shoot_fp64(a, s, row0, row1);
         } else if (split > kMaxClusterSplit) {
             // partials of up to kGsplitBytes per pass (at least one tile row), in a
@@ -531,7 +532,7 @@ int mlens_trace(mlens_ctx *ctx, const double *theta, int64_t k, double *beta, vo
     double2 *d = nullptr;
     MLENS_CUDA(dmalloc(&d, (size_t)k * 2 * sizeof(double2)), "cudaMalloc(trace)");
     cudaError_t e = cudaMemcpyAsync(d, theta, (size_t)k * sizeof(double2), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = launch_trace_fp64(ctx->d_stars, ctx->n_pad, ctx->lens, d, d + k, k, s);
+    if (e == cudaSuccess) e = launch_trace_fp64(ctx->d_stars, ctx->n, ctx->lens, d, d + k, k, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(beta, d + k, (size_t)k * sizeof(double2), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     dfree(d);
