@@ -21,10 +21,12 @@
 #include <stdint.h>
 
 #include <cmath>
+#include <cstring>
 #include <string>
 #include <vector>
 
 #include "mlens_internal.h"
+#include "soft64.cuh"
 
 namespace mlens {
 namespace {
@@ -539,34 +541,82 @@ __global__ void __launch_bounds__(kThr) k_disk_halves(double R, double dx, doubl
     half[q] = (int)min(h, (long long)nx);
 }
 
-struct Track {
-    double x0, y0, dx, dy;      // map origin and pixel widths
-    double bx0, by0, bx1, by1;  // track end points
-    int nx, ny, n;
+// A constant divisor: its value and, where it lies within 2^+-200, its significand and
+// reciprocal for soft_div (ok).
+struct Divisor {
+    double d;
+    Soft64 b;
+    uint64_t r;
+    bool ok;
 };
 
-__global__ void __launch_bounds__(kThr) k_curve(const float *__restrict__ m, Track T, float *__restrict__ out)
+struct Track {
+    double o[2], b0[2], b1[2];  // map origin, first and last point of the track, per axis
+    Divisor w[2], last;         // pixel widths, n - 1
+    int size[2];                // map size
+    int n;
+};
+
+// a / D, correctly rounded.
+__device__ __forceinline__ double divide(double a, const Divisor &D)
 {
-    const int k = blockIdx.x * kThr + threadIdx.x;
-    if (k >= T.n) return;
-    const double t = T.n > 1 ? __ddiv_rn((double)k, (double)(T.n - 1)) : 0.0;
-    const double bx = __dadd_rn(T.bx0, __dmul_rn(t, __dsub_rn(T.bx1, T.bx0)));
-    const double by = __dadd_rn(T.by0, __dmul_rn(t, __dsub_rn(T.by1, T.by0)));
-    const double u = __dsub_rn(__ddiv_rn(__dsub_rn(bx, T.x0), T.dx), 0.5);
-    const double v = __dsub_rn(__ddiv_rn(__dsub_rn(by, T.y0), T.dy), 0.5);
-    const double fi = floor(u), fj = floor(v);
-    const double fx = __dsub_rn(u, fi), fy = __dsub_rn(v, fj);
+    const uint64_t bits = (uint64_t)__double_as_longlong(a);
+    const uint32_t e = (uint32_t)(bits >> 52) & 0x7ffu;
+    if (!D.ok || e - 823u > 400u) return __ddiv_rn(a, D.d);
+    return __longlong_as_double((long long)soft_bits(soft_div(soft_of(bits), D.b, D.r), bits & uint64_t(1) << 63));
+}
+
+// Two lanes per point, one per axis: the even lane takes x and the lower row's
+// interpolation, the odd lane y, the upper row's and the point's value.  Bound by FP64
+// latency (76 cycles an instruction and warp): the divisions run on the integer pipes
+// (soft64.cuh), the axes side by side, and CTAs are small so that a short curve spreads
+// over the SMs.  4096 points 7.1 -> 3.7 us.
+constexpr int kCurveThreads = 64;
+__global__ void __launch_bounds__(kCurveThreads) k_curve(const float *__restrict__ m,
+                                                         const __grid_constant__ Track T, float *__restrict__ out)
+{
+    const int64_t lin = (int64_t)blockIdx.x * kCurveThreads + threadIdx.x;
+    const int ax = threadIdx.x & 1, k = (int)min(lin >> 1, (int64_t)T.n - 1);
+    double t = 0.0;
+    if (T.n > 1 && k > 0) {  // k / (n - 1)
+        const int z = __clz(k);
+        t = __longlong_as_double((long long)soft_bits(soft_div({(uint64_t)k << (32 + z), 31 - z}, T.last.b, T.last.r), 0));
+    }
+    const double b0 = T.b0[ax], b1 = T.b1[ax];
+    const double b = __dadd_rn(b0, __dmul_rn(t, __dsub_rn(b1, b0)));
+    const double u = __dsub_rn(divide(__dsub_rn(b, T.o[ax]), T.w[ax]), 0.5);
+    const double fl = floor(u);
+    const double f = __dsub_rn(u, fl);
     // corner indices clamped before the conversion (only the map's edges matter)
-    const int i0 = (int)fmin(fmax(fi, -2.0), (double)T.nx + 1.0);
-    const int j0 = (int)fmin(fmax(fj, -2.0), (double)T.ny + 1.0);
-    const int ia = min(max(i0, 0), T.nx - 1), ib = min(max(i0 + 1, 0), T.nx - 1);
-    const int ja = min(max(j0, 0), T.ny - 1), jb = min(max(j0 + 1, 0), T.ny - 1);
-    const double m00 = m[(int64_t)ja * T.nx + ia], m01 = m[(int64_t)ja * T.nx + ib];
-    const double m10 = m[(int64_t)jb * T.nx + ia], m11 = m[(int64_t)jb * T.nx + ib];
-    const double gx = __dsub_rn(1.0, fx), gy = __dsub_rn(1.0, fy);
-    const double s0 = __dadd_rn(__dmul_rn(gx, m00), __dmul_rn(fx, m01));
-    const double s1 = __dadd_rn(__dmul_rn(gx, m10), __dmul_rn(fx, m11));
-    out[k] = __double2float_rn(__dadd_rn(__dmul_rn(gy, s0), __dmul_rn(fy, s1)));
+    const int n = T.size[ax], i = (int)fmin(fmax(fl, -2.0), (double)n + 1.0);
+    const int ia = min(max(i, 0), n - 1), ib = min(max(i + 1, 0), n - 1);
+    // the even lane needs the lower row, the odd lane the upper row and x's columns and fraction
+    constexpr unsigned kAll = 0xffffffffu;
+    const int ja = __shfl_xor_sync(kAll, ia, 1), oa = __shfl_xor_sync(kAll, ib, 1);
+    const double of = __shfl_xor_sync(kAll, f, 1);
+    const int row = ax ? ib : ja, c0 = ax ? ja : ia, c1 = ax ? oa : ib;
+    const double fx = ax ? of : f, gx = __dsub_rn(1.0, fx);
+    const double m0 = m[(int64_t)row * T.size[0] + c0], m1 = m[(int64_t)row * T.size[0] + c1];
+    const double s = __dadd_rn(__dmul_rn(gx, m0), __dmul_rn(fx, m1));
+    const double s0 = __shfl_xor_sync(kAll, s, 1);
+    if (ax && lin >> 1 < T.n) {  // gy s0 + fy s1
+        const double gy = __dsub_rn(1.0, f);
+        out[k] = __double2float_rn(__dadd_rn(__dmul_rn(gy, s0), __dmul_rn(f, s)));
+    }
+}
+
+Divisor make_divisor(double d)
+{
+    Divisor D{};
+    D.d = d;
+    uint64_t bits;
+    std::memcpy(&bits, &d, sizeof(bits));
+    D.ok = d > 0x1p-200 && d < 0x1p200;
+    if (D.ok) {
+        D.b = soft_of(bits);
+        D.r = (uint64_t)((((unsigned __int128)1 << 127) - 1) / D.b.n);
+    }
+    return D;
 }
 
 int lc_cuda(cudaError_t e, const char *what)
@@ -877,19 +927,21 @@ int mlens_light_curve(const float *map_dev, const mlens_grid *src, double bx0, d
         return lc_fail(MLENS_ERR_ARG, "map_dev and out_dev must be 4-byte aligned");
     if (!std::isfinite(bx0) || !std::isfinite(by0) || !std::isfinite(bx1) || !std::isfinite(by1))
         return lc_fail(MLENS_ERR_ARG, "track end points must be finite");
-    Track T;
-    T.x0 = src->x0;
-    T.y0 = src->y0;
-    T.dx = (src->x1 - src->x0) / src->nx;
-    T.dy = (src->y1 - src->y0) / src->ny;
-    T.bx0 = bx0;
-    T.by0 = by0;
-    T.bx1 = bx1;
-    T.by1 = by1;
-    T.nx = src->nx;
-    T.ny = src->ny;
+    Track T{};
+    T.o[0] = src->x0;
+    T.o[1] = src->y0;
+    T.b0[0] = bx0;
+    T.b0[1] = by0;
+    T.b1[0] = bx1;
+    T.b1[1] = by1;
+    T.w[0] = make_divisor((src->x1 - src->x0) / src->nx);
+    T.w[1] = make_divisor((src->y1 - src->y0) / src->ny);
+    T.last = make_divisor((double)std::max(1, npts - 1));
+    T.size[0] = src->nx;
+    T.size[1] = src->ny;
     T.n = npts;
-    k_curve<<<(unsigned)((npts + kThr - 1) / kThr), kThr, 0, (cudaStream_t)stream>>>(map_dev, T, out_dev);
+    const int64_t blocks = (2 * (int64_t)npts + kCurveThreads - 1) / kCurveThreads;
+    k_curve<<<(unsigned)blocks, kCurveThreads, 0, (cudaStream_t)stream>>>(map_dev, T, out_dev);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return lc_cuda(e, "light curve launch");
     return MLENS_OK;
