@@ -137,6 +137,8 @@ SIGNATURES = {
 def load(path: Optional[str] = None):
     """Open libmlens.so (built by build.py) and declare its signatures."""
     global _lib
+    if _lib is not None and path is None:
+        return _lib
     with _lock:
         if _lib is not None and path is None:
             return _lib
@@ -190,10 +192,25 @@ def grid(g) -> mlens_grid:
     return mlens_grid(float(x0), float(x1), float(y0), float(y1), int(nx), int(ny))
 
 
+_raw_stream = None  # () -> the current device's current stream as an address
+
+
+def _current_stream() -> int:
+    """torch's current stream on the current device, without building a Stream object
+    for every call (2 us of a light curve's 11)."""
+    global _raw_stream
+    if _raw_stream is None:
+        import torch
+        s = torch.cuda.current_stream().cuda_stream  # initialises CUDA
+        get, dev = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+        _raw_stream = (lambda: get(dev())) if get and dev else (lambda: torch.cuda.current_stream().cuda_stream)
+        return s
+    return _raw_stream()
+
+
 def _stream_ptr(stream):
     if stream is None:
-        import torch
-        return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+        return C.c_void_p(_current_stream())
     if hasattr(stream, "cuda_stream"):
         return C.c_void_p(stream.cuda_stream)
     return C.c_void_p(int(stream))
