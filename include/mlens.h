@@ -105,7 +105,8 @@ int mlens_set_precision(mlens_ctx *ctx, int32_t precision);
  * mlens_set_tuning -- launch shape of the FP32 kernels for later calls on this
  * context: rays_per_thread in {4, 8} (tile 64 x 16 or 64 x 32 rays per CTA of
  * 256 threads), star_stage in {128, 256, 512} stars staged through shared
- * memory at a time (0 = 256; 512 is accepted and staged as 256), and fma_pairs in {0, 1}: 0 takes every
+ * memory at a time (0 = 256; the kernels now stage 128 whatever the setting, which
+ * still decides whether the star sum may be split), and fma_pairs in {0, 1}: 0 takes every
  * reciprocal 1/r^2 from the MUFU unit (16 per SM per clock, the bound of the
  * direct sum); 1 takes a share of them (a thread's first ray pair on every third
  * star, 7.8 %) from Newton-Raphson iterations on the FMA pipe instead, which
@@ -381,7 +382,7 @@ int mlens_batch_set_tuning(mlens_batch *b, int32_t rays_per_thread, int32_t star
 
 /*
  * mlens_batch_tune -- the autotuner: time the launch shapes (rays per thread 8
- * or 4, star stage 256 or 128, fma_pairs 0 or 1) on this batch (a warm-up and
+ * or 4, fma_pairs 0 or 1) on this batch (a warm-up and
  * two timed replays each, CUDA events on `stream`), keep the fastest and report
  * it (any output pointer may be NULL; *best_ms = -1 when the shape came from the
  * cache).  Results are cached per process by device and workload

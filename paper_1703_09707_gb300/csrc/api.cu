@@ -135,6 +135,18 @@ int read_stats(unsigned long long *d_stats, uint64_t total, mlens_stats *st, cud
     return MLENS_OK;
 }
 
+// The map (unless the call accumulates) and the three ray counters to zero, one launch.
+cudaError_t clear_map(uint32_t *counts, const mlens_grid *src, uint32_t flags, unsigned long long *stats,
+                      cudaStream_t s)
+{
+    ClearArgs c{};
+    c.map = counts;
+    c.n = flags & MLENS_ACCUMULATE ? 0 : (size_t)src->nx * (size_t)src->ny;
+    c.words[0] = reinterpret_cast<uint32_t *>(stats);
+    c.nwords[0] = 6;
+    return launch_clear(c, s);
+}
+
 // Ray rows per tile of the FP32 kernels (the FP64 kernel's 4-row blocks divide it).
 int tile_rows_of(const mlens_ctx *ctx) { return 8 * ctx->pairs_per_thread; }
 
@@ -168,13 +180,11 @@ int shoot_impl(mlens_ctx *ctx, const mlens_grid *rays, const mlens_grid *src, ui
     if (flags & ~MLENS_ACCUMULATE) return fail(MLENS_ERR_ARG, "unknown flag bits");
     if ((rc = check_current_device(ctx->device))) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t npix = (size_t)src->nx * (size_t)src->ny;
-    if (!(flags & MLENS_ACCUMULATE))
-        MLENS_CUDA(cudaMemsetAsync(counts, 0, npix * sizeof(uint32_t), s), "cudaMemsetAsync(counts)");
-    MLENS_CUDA(cudaMemsetAsync(ctx->d_stats, 0, 3 * sizeof(unsigned long long), s), "cudaMemsetAsync(stats)");
+    MLENS_CUDA(clear_map(counts, src, flags, ctx->d_stats, s), "clear launch");
     ShootArgs a{};
     a.stars = ctx->d_stars;
     a.nstars = ctx->n_pad;
+    a.n = ctx->n;
     a.rays = make_ray_grid(*rays);
     a.bin = make_bin_grid(*src);
     a.lens = ctx->lens;
@@ -209,7 +219,7 @@ int shoot_impl(mlens_ctx *ctx, const mlens_grid *rays, const mlens_grid *src, ui
             e = launch_shoot_split(a, ctx->pairs_per_thread, split, s, ty0, ty1, ctx->fma_pairs);
         } else {
             e = launch_shoot_fp32(a, ctx->pairs_per_thread, ctx->precision == MLENS_PREC_FP32_NAIVE, s,
-                                  ctx->star_stage, ctx->fma_pairs, ty0, ty1);
+                                  ctx->fma_pairs, ty0, ty1, true);
         }
     }
     if (e != cudaSuccess) return cuda_fail(e, "shoot kernel launch");
@@ -376,10 +386,7 @@ int bin_impl(const void *beta_dev, int64_t n, int rnx, int rny, const mlens_grid
     unsigned long long *st = nullptr;
     if ((rc = device_scratch(&st))) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    const size_t npix = (size_t)src->nx * (size_t)src->ny;
-    if (!(flags & MLENS_ACCUMULATE))
-        MLENS_CUDA(cudaMemsetAsync(counts_dev, 0, npix * sizeof(uint32_t), s), "cudaMemsetAsync(counts)");
-    MLENS_CUDA(cudaMemsetAsync(st, 0, 3 * sizeof(unsigned long long), s), "cudaMemsetAsync(stats)");
+    MLENS_CUDA(clear_map(counts_dev, src, flags, st, s), "clear launch");
     BinArgs a{};
     a.beta = reinterpret_cast<const float4 *>(beta_dev);
     a.n = n;

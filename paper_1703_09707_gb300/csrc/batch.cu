@@ -2,7 +2,7 @@
 // a grid of simulations over (<M*>, gamma, kappa_*, kappa_c), each its own map),
 // replayed as a CUDA graph, with an autotuner for the launch shape.
 //
-// The work queue holds one item per (field, ray tile); fields are ordered by the
+// The work queue holds one item per (field, half ray tile); fields are ordered by the
 // cost of one tile (stars x rays per tile), heaviest first, so the last items
 // handed out are the cheapest and CTAs finish together (longest-processing-time
 // ordering).  The graph holds the map clears, the counter clears and the
@@ -91,7 +91,7 @@ int build_tables(mlens_batch *b)
     const int nf = b->nfields;
     std::vector<int64_t> tiles(nf), cost(nf);
     for (int f = 0; f < nf; ++f) {
-        tiles[f] = tiles_of(b->h_fields[f].rays, b->pairs_per_thread);
+        tiles[f] = 2 * tiles_of(b->h_fields[f].rays, b->pairs_per_thread);  // half tiles
         cost[f] = std::max<int64_t>(b->n_pad[f], 1);
     }
     std::vector<int> order(nf);
@@ -103,7 +103,7 @@ int build_tables(mlens_batch *b)
     BCUDA(cudaMemcpy(b->d_order, order.data(), sizeof(int) * nf, cudaMemcpyHostToDevice), "cudaMemcpy(order)");
     BCUDA(cudaMemcpy(b->d_begin, begin.data(), sizeof(int64_t) * (nf + 1), cudaMemcpyHostToDevice),
           "cudaMemcpy(begin)");
-    BCUDA(batch_grid_size(b->pairs_per_thread, b->star_stage, &b->grid, b->fma_pairs), "occupancy query");
+    BCUDA(batch_grid_size(b->pairs_per_thread, &b->grid, b->fma_pairs), "occupancy query");
     return MLENS_OK;
 }
 
@@ -125,7 +125,7 @@ int capture(mlens_batch *b)
             e = cudaMemsetAsync(b->counts[f], 0, (size_t)b->srcs[f].nx * b->srcs[f].ny * sizeof(uint32_t), b->cap);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_stats, 0, sizeof(unsigned long long) * 3 * b->nfields, b->cap);
     if (e == cudaSuccess) e = cudaMemsetAsync(b->d_counter, 0, sizeof(unsigned long long), b->cap);
-    if (e == cudaSuccess) e = launch_shoot_batch(L, b->pairs_per_thread, b->star_stage, b->cap, b->fma_pairs);
+    if (e == cudaSuccess) e = launch_shoot_batch(L, b->pairs_per_thread, b->cap, b->fma_pairs);
     cudaGraph_t g = nullptr;
     cudaError_t e2 = cudaStreamEndCapture(b->cap, &g);
     if (e != cudaSuccess) {
@@ -252,6 +252,7 @@ int mlens_batch_create(mlens_batch **out, mlens_ctx *const *ctxs, int32_t nfield
         ShootArgs a{};
         a.stars = ctxs[f]->d_stars;
         a.nstars = ctxs[f]->n_pad;
+        a.n = ctxs[f]->n;
         a.rays = make_ray_grid(rays[f]);
         a.bin = make_bin_grid(srcs[f]);
         a.lens = ctxs[f]->lens;
@@ -330,17 +331,17 @@ int mlens_batch_tune(mlens_batch *b, void *stream, int32_t *rays_per_thread, int
         }
     }
     const int cand_rpt[2] = {8, 4};
-    const int cand_st[2] = {256, 128};
     cudaEvent_t e0, e1;
     BCUDA(cudaEventCreate(&e0), "cudaEventCreate");
     BCUDA(cudaEventCreate(&e1), "cudaEventCreate");
     double best = 1e300;
-    int brpt = 8, bst = 256, bfm = 0;
+    int brpt = 8, bfm = 0;
+    const int bst = 256;  // the kernels stage alike whatever the setting
     int rc = MLENS_OK;
-    for (int c = 0; c < 8 && rc == MLENS_OK; ++c) {
-        const int i = (c / 2) % 2, j = c % 2, fm = c / 4;
+    for (int c = 0; c < 4 && rc == MLENS_OK; ++c) {
+        const int i = c % 2, fm = c / 2;
         {
-            if ((rc = set_shape(b, cand_rpt[i], cand_st[j], fm)) != MLENS_OK) break;
+            if ((rc = set_shape(b, cand_rpt[i], bst, fm)) != MLENS_OK) break;
             if ((rc = mlens_batch_run(b, nullptr, stream)) != MLENS_OK) break;  // warm-up + capture
             double tmin = 1e300;
             for (int r = 0; r < 2; ++r) {
@@ -359,7 +360,6 @@ int mlens_batch_tune(mlens_batch *b, void *stream, int32_t *rays_per_thread, int
             if (rc == MLENS_OK && tmin < best) {
                 best = tmin;
                 brpt = cand_rpt[i];
-                bst = cand_st[j];
                 bfm = fm;
             }
         }

@@ -67,9 +67,10 @@ __device__ __forceinline__ void bin_block(const BinArgs &a)
     const float4 vc = *centre;
     hist_zero(hist);
     if (tid == 0) sred[0] = sred[1] = sred[2] = 0u;
-    const WinHist W = make_window(hist, win_origin(pair_axis_rough(vc.x, a.bin.ax), a.bin.nx),
+    const WinHist<> W = make_window(hist, win_origin(pair_axis_rough(vc.x, a.bin.ax), a.bin.nx),
                                   win_origin(pair_axis_rough(vc.y, a.bin.ay), a.bin.ny), a.bin);
     __syncthreads();
+    pdl_wait();  // the map's and the counters' clears
     unsigned no = 0, nn = 0;
 #pragma unroll
     for (int r0 = 0; r0 < kBinCnt; r0 += kBinPer) {
@@ -92,13 +93,11 @@ cudaError_t launch_bin(const BinArgs &a, cudaStream_t s)
     if (a.rnx > 0) {
         const int64_t tx = (a.rnx + kBinTileX - 1) / kBinTileX, ty = (a.rny + kBinTileY - 1) / kBinTileY;
         if (tx > 0x7fffffff || ty > 65535) return cudaErrorInvalidConfiguration;
-        k_bin_grid<<<dim3((unsigned)tx, (unsigned)ty), kBinThreads, 0, s>>>(a);
-        return cudaGetLastError();
+        return launch_pdl(k_bin_grid, dim3((unsigned)tx, (unsigned)ty), dim3(kBinThreads), 0, s, a);
     }
     const int64_t nb = (a.n + kBinRecs - 1) / kBinRecs;
     if (nb > 0x7fffffff) return cudaErrorInvalidConfiguration;
-    k_bin_flat<<<(unsigned)nb, kBinThreads, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k_bin_flat, dim3((unsigned)nb), dim3(kBinThreads), 0, s, a);
 }
 
 }  // namespace mlens

@@ -416,15 +416,6 @@ cudaError_t ff_init_params(float *params, float *z, int nrc, uint64_t seed, cuda
     return cudaGetLastError();
 }
 
-// Programmatic dependent launch between the training steps' kernels: a kernel
-// launched with programmatic stream serialisation may begin while the one before
-// it finishes; pdl_wait() returns once that one has completed and its writes are
-// visible, and pdl_launch_next() lets the next kernel begin launching once every
-// CTA of this one has called it.  Both do nothing in a kernel launched without
-// the attribute.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // ===================================================== training kernel
 constexpr int kWaitPolls = 1 << 20;  // bound on a tensor-core completion wait
 constexpr int kProbePolls = 1024;    // bound on a probe wait (an mbarrier nothing arrives on)
@@ -1043,24 +1034,6 @@ __global__ void __launch_bounds__(256, 2) k_ff_train(TrainArgs A)
     if (tid < 32) umma::tmem_dealloc(tm, L::ncols);
 }
 
-// Launch with programmatic stream serialisation (PDL): the kernel may begin while
-// the previous one of the stream finishes (see pdl_wait).
-template <class... P, class... A>
-static cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
-{
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k, args...);
-}
-
 cudaError_t ff_train_step(const TrainArgs &t, int64_t nsamples, cudaStream_t s, bool pdl)
 {
     // two CTAs of ~85 KB per SM (tensor memory allows no more): the largest shared-memory carveout
@@ -1281,7 +1254,10 @@ constexpr int kNearChunk = NET ? 4 : 2;
 constexpr int kTcChunk = 128;                            // rays per tensor-core MMA (M)
 constexpr int kTcABytes = kTcChunk * kHid * 2;           // one warpgroup's A operand (16 KB)
 constexpr int kTcSmem = 2 * kTcABytes;                   // the two A operands
-using LearnTileSmem = ShootSmem<4, 256, true>;           // the near-field star stage, then the window
+union LearnTileSmem {  // the near-field star stage, then the window
+    StarStage<256> st;
+    uint32_t hist[kWin * kWin];
+};
 constexpr size_t kLearnedDynSmem = kTcSmem > sizeof(LearnTileSmem) ? kTcSmem : sizeof(LearnTileSmem);
 
 // LO: the ray offsets carry low parts (grids whose offsets are not exact floats,
@@ -1608,12 +1584,12 @@ __device__ __forceinline__ void learned_tile(const LearnedArgs &L, int bx, int b
     const bool col_ok = ix < R.nx;
     __syncthreads();
     hist_zero(sm.hist);
-    if (tid == 0) {
+    if (tid == kThreads / 2 + kTileX / 2) {  // the tile's middle ray
         ts.win[0] = win_origin(pair_axis_rough(bxh[0], a.bin.ax), a.bin.nx);
         ts.win[1] = win_origin(pair_axis_rough(byh[0], a.bin.ay), a.bin.ny);
     }
     __syncthreads();
-    const WinHist W = make_window(sm.hist, ts.win[0], ts.win[1], a.bin);
+    const WinHist<> W = make_window(sm.hist, ts.win[0], ts.win[1], a.bin);
     const int nrow = col_ok ? min(2 * NP, R.ny - (j0 + tg * 2 * NP)) : 0;  // this thread's rays in the grid
     unsigned no = 0, nn = 0;
 #pragma unroll

@@ -490,14 +490,20 @@ int mlens_shoot_learned(mlens_ctx *ctx, const mlens_grid *rays, const mlens_grid
         nitems = (int64_t)sub.size();
         nrows_total = (int64_t)rays->nx * (row_end - row_begin);
     }
-    if (!(flags & MLENS_ACCUMULATE))
-        FCUDA(cudaMemsetAsync(counts_dev, 0, (size_t)src->nx * src->ny * sizeof(uint32_t), s), "memset(counts)");
-    FCUDA(cudaMemsetAsync(ctx->d_stats, 0, 3 * sizeof(unsigned long long), s), "memset(stats)");
-    FCUDA(cudaMemsetAsync(f->counter, 0, sizeof(unsigned long long), s), "memset(counter)");
-    FCUDA(cudaMemsetAsync(f->d_err, 0, sizeof(int), s), "memset(err)");
+    ClearArgs clr{};
+    clr.map = counts_dev;
+    clr.n = flags & MLENS_ACCUMULATE ? 0 : (size_t)src->nx * (size_t)src->ny;
+    clr.words[0] = reinterpret_cast<uint32_t *>(ctx->d_stats);
+    clr.nwords[0] = 6;
+    clr.words[1] = reinterpret_cast<uint32_t *>(f->counter);
+    clr.nwords[1] = 2;
+    clr.words[2] = reinterpret_cast<uint32_t *>(f->d_err);
+    clr.nwords[2] = 1;
+    FCUDA(launch_clear(clr, s), "clear launch");
     LearnedArgs L{};
     L.plain.stars = ctx->d_stars;
     L.plain.nstars = ctx->n_pad;
+    L.plain.n = ctx->n;
     L.plain.rays = make_ray_grid(*rays);
     L.plain.bin = make_bin_grid(*src);
     L.plain.lens = ctx->lens;

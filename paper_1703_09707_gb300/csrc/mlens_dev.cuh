@@ -11,6 +11,14 @@
 
 namespace mlens {
 
+// Programmatic dependent launch: a kernel launched with programmatic stream
+// serialisation may begin while the one before it finishes; pdl_wait() returns once that
+// one has completed and its writes are visible, and pdl_launch_next() lets the next
+// kernel begin launching once every CTA of this one has called it.  Both do nothing in a
+// kernel launched without the attribute.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ------------------------------------------------------------ float pairs
 // Knuth's error-free TwoSum: s + e == a + b exactly, s = fl(a + b).
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
@@ -122,30 +130,36 @@ __device__ __forceinline__ int pair_axis_rough(float bh, const AxisPair &A)
 // them land in a small patch of the source map.  The CTA counts that patch in
 // a W x W shared-memory window (placed around the pixel of one of its rays, inside the
 // map) and adds the window to the global map at the end; rays outside the window go
-// straight to global atomics.  One atomic per ray: the shared-memory increment merges
+// straight to global atomics.  W is 64, or 32 for the direct sum's half tiles.  One atomic per ray: the shared-memory increment merges
 // a warp's equal pixels in hardware, which cost less than finding runs of equal
 // pixels with a shuffle, a vote and a branch per ray.
 constexpr int kWin = 64;
 
+template <int W = kWin>
 struct WinHist {
-    uint32_t *h;         // kWin*kWin counters in shared memory
+    uint32_t *h;         // W*W counters in shared memory
     int wx0, wy0;        // window origin in pixels, within the map
-    unsigned nwx, nwy;   // window extent: kWin, or the map's where that is smaller
+    unsigned nwx, nwy;   // window extent: W, or the map's where that is smaller
 };
 
 // Origin of the window on one axis, for a window centred on pixel p.
-__device__ __forceinline__ int win_origin(int p, int n) { return min(max(p - kWin / 2, 0), max(n - kWin, 0)); }
-
-__device__ __forceinline__ WinHist make_window(uint32_t *h, int wx0, int wy0, const BinGrid &g)
+template <int W = kWin>
+__device__ __forceinline__ int win_origin(int p, int n)
 {
-    return {h, wx0, wy0, (unsigned)min(kWin, g.nx), (unsigned)min(kWin, g.ny)};
+    return min(max(p - W / 2, 0), max(n - W, 0));
+}
+
+template <int W = kWin>
+__device__ __forceinline__ WinHist<W> make_window(uint32_t *h, int wx0, int wy0, const BinGrid &g)
+{
+    return {h, wx0, wy0, (unsigned)min(W, g.nx), (unsigned)min(W, g.ny)};
 }
 
 // One float-pair beta into the histogram; counts it in `out` (finite, outside the map)
 // or `nan` otherwise.
-template <bool NORM>
-__device__ __forceinline__ void bin_pair(float xh, float yh, float xl, float yl, const BinGrid &g, const WinHist &W,
-                                         uint32_t *counts, unsigned &out, unsigned &nan)
+template <bool NORM, int WN>
+__device__ __forceinline__ void bin_pair(float xh, float yh, float xl, float yl, const BinGrid &g,
+                                         const WinHist<WN> &W, uint32_t *counts, unsigned &out, unsigned &nan)
 {
     int px, py;
     if (!fast_pixel<NORM>(xh, yh, xl, yl, g.fast, px, py)) {
@@ -159,7 +173,7 @@ __device__ __forceinline__ void bin_pair(float xh, float yh, float xl, float yl,
     }
     const unsigned wx = (unsigned)(px - W.wx0), wy = (unsigned)(py - W.wy0);
     if (wx < W.nwx && wy < W.nwy)
-        atomicAdd(&W.h[wy * kWin + wx], 1u);
+        atomicAdd(&W.h[wy * WN + wx], 1u);
     else if ((unsigned)px < (unsigned)g.nx && (unsigned)py < (unsigned)g.ny)
         atomicAdd(&counts[py * g.nx + px], 1u);
     else
@@ -167,20 +181,22 @@ __device__ __forceinline__ void bin_pair(float xh, float yh, float xl, float yl,
 }
 
 // Clear the window (uint4 stores; the window is 16-byte aligned).
+template <int W = kWin>
 __device__ __forceinline__ void hist_zero(uint32_t *h)
 {
     uint4 *h4 = reinterpret_cast<uint4 *>(h);
-    for (int b = threadIdx.x; b < kWin * kWin / 4; b += blockDim.x) h4[b] = make_uint4(0u, 0u, 0u, 0u);
+    for (int b = threadIdx.x; b < W * W / 4; b += blockDim.x) h4[b] = make_uint4(0u, 0u, 0u, 0u);
 }
 
 // Add the window to the global map (bins outside the map are never filled).
-__device__ __forceinline__ void hist_flush(const WinHist &W, const BinGrid &g, uint32_t *counts)
+template <int WN>
+__device__ __forceinline__ void hist_flush(const WinHist<WN> &W, const BinGrid &g, uint32_t *counts)
 {
     const uint4 *h4 = reinterpret_cast<const uint4 *>(W.h);
-    for (int b = threadIdx.x; b < kWin * kWin / 4; b += blockDim.x) {
+    for (int b = threadIdx.x; b < WN * WN / 4; b += blockDim.x) {
         const uint4 v = h4[b];
         if ((v.x | v.y | v.z | v.w) == 0u) continue;
-        const int64_t base = (int64_t)(W.wy0 + b / (kWin / 4)) * g.nx + (W.wx0 + 4 * (b % (kWin / 4)));
+        const int64_t base = (int64_t)(W.wy0 + b / (WN / 4)) * g.nx + (W.wx0 + 4 * (b % (WN / 4)));
         if (v.x) atomicAdd(&counts[base + 0], v.x);
         if (v.y) atomicAdd(&counts[base + 1], v.y);
         if (v.z) atomicAdd(&counts[base + 2], v.z);

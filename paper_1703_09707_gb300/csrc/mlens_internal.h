@@ -63,13 +63,14 @@ struct LensTerms {
 struct ShootArgs {
     const float4 *stars;    // (x, y, m, 0), padded
     int64_t nstars;         // padded count, multiple of kStarPad
+    int64_t n;              // of which stars given
     RayGrid rays;
     BinGrid bin;
     LensTerms lens;
     uint32_t *counts;
     unsigned long long *stats;  // [binned, out, nan]
     void *beta_out;         // nullable: float4 pairs or double2 (FP64)
-    float4 *gpart;          // global split: 2 NP float4 per thread per (tile, slice) (launch_shoot_gsplit)
+    float4 *gpart;          // global split: 2 NP float4 per thread per (half tile, slice) (launch_shoot_gsplit)
     int gslices;            // global split: slices per tile
 };
 
@@ -89,7 +90,7 @@ struct BatchLaunch {
     const int *order;             // field processing order, heaviest first (device)
     const int64_t *begin;         // nfields+1 item offsets in that order (device)
     int nfields;
-    int64_t total;                // total (field, tile) items
+    int64_t total;                // total (field, half tile) items
     unsigned long long *counter;  // work-queue counter, zero before each launch (device)
 };
 
@@ -105,23 +106,52 @@ inline cudaError_t allow_dynamic_smem(K kernel, size_t bytes)
     return e;
 }
 
+// Zero words before a call's kernel (clear.cu): a map of n words (n = 0: none) and up
+// to three short runs of words.
+struct ClearArgs {
+    uint32_t *map;
+    size_t n;
+    uint32_t *words[3];
+    int nwords[3];
+};
+cudaError_t launch_clear(const ClearArgs &a, cudaStream_t s);
+
+// Launch with programmatic stream serialisation (PDL): the kernel may begin while the
+// previous one of the stream finishes (pdl_wait in mlens_dev.cuh).
+template <class... P, class... A>
+inline cudaError_t launch_pdl(void (*k)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // launchers (defined in the .cu files)
-// pairs_per_thread in {2, 4} (4 or 8 rays per thread); stage in {128, 256, 512} stars (512 runs as 256)
+// pairs_per_thread in {2, 4} (4 or 8 rays per thread)
 // fma_pairs in {0, 1}: 1 takes a share of the reciprocals (pair 0 on every third
 // star, 7.8 %) from the FMA pipe, 0 every reciprocal from the MUFU unit
+// pdl: the launch before it on the stream is launch_clear's, which the kernel overlaps
 // [ty0, ty1): the tile rows to shoot (tile_rows(pairs_per_thread) ray rows each;
 // ty1 < 0 = through the last)
 cudaError_t launch_shoot_fp32(const ShootArgs &a, int pairs_per_thread, bool naive, cudaStream_t s,
-                              int stage = 256, int fma_pairs = 0, int ty0 = 0, int ty1 = -1);
-cudaError_t launch_shoot_batch(const BatchLaunch &b, int pairs_per_thread, int stage, cudaStream_t s,
-                               int fma_pairs = 0);
-cudaError_t batch_grid_size(int pairs_per_thread, int stage, int *grid, int fma_pairs = 0);
+                              int fma_pairs = 0, int ty0 = 0, int ty1 = -1, bool pdl = false);
+cudaError_t launch_shoot_batch(const BatchLaunch &b, int pairs_per_thread, cudaStream_t s, int fma_pairs = 0);
+cudaError_t batch_grid_size(int pairs_per_thread, int *grid, int fma_pairs = 0);
 int64_t tiles_of(const RayGrid &r, int pairs_per_thread);
+__host__ __device__ inline int halves_x(const RayGrid &r) { return 2 * ((r.nx + 63) / 64); }  // half tiles per tile row
 // ray rows [row0, row1) (row0 a multiple of 4; row1 < 0 = through the last)
 cudaError_t launch_shoot_fp64(const ShootArgs &a, cudaStream_t s, int row0 = 0, int row1 = -1);
 cudaError_t launch_trace_fp64(const float4 *stars, int64_t nstars, const LensTerms &lens, const double2 *theta,
                               double2 *beta, int64_t k, cudaStream_t s);
-// Split star sum (shoot_split.cu; re-centred FP32, 256-star stages, either
+// Split star sum (shoot_split.cu; re-centred FP32, the default star stage, either
 // reciprocal split): clusters of `split` in 2 .. 8 CTAs per tile.  auto_star_split
 // picks the split for a grid (1 = none) from the wave efficiency on `nsm` SMs.
 constexpr int kSplitStage = 256;
@@ -148,7 +178,7 @@ cudaError_t launch_shoot_gsplit(const ShootArgs &a, int pairs_per_thread, int sp
 cudaError_t launch_shoot_split_list(const ShootArgs &a, const int *tiles, int64_t ntiles, int split, cudaStream_t s,
                                     int fma_pairs);
 int fallback_star_split(int64_t nstars);
-cudaError_t launch_bin(const BinArgs &a, cudaStream_t s);
+cudaError_t launch_bin(const BinArgs &a, cudaStream_t s);  // after launch_clear on the same stream
 
 // helpers (api.cu)
 void set_last_error(const std::string &msg);

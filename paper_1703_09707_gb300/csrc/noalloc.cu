@@ -118,13 +118,14 @@ extern "C" int mlens_shoot_noalloc(const void *stars_dev, int64_t n, double kapp
     ShootArgs a{};
     a.stars = sc->stars;
     a.nstars = npad;
+    a.n = n;
     a.rays = make_ray_grid(*rays);
     a.bin = make_bin_grid(*src);
     a.lens = make_lens_terms(kappa_c, gamma1, gamma2);
     a.counts = counts_dev;
     a.stats = sc->stats;
     a.beta_out = nullptr;
-    if ((e = launch_shoot_fp32(a, 4, false, s, 256, kDefaultFmaPairs)) != cudaSuccess)
+    if ((e = launch_shoot_fp32(a, 4, false, s, kDefaultFmaPairs)) != cudaSuccess)
         return cuda_error(e, "no-alloc shoot kernel launch");
     if (stats_host) {
         unsigned long long h[3];

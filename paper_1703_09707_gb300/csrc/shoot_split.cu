@@ -24,64 +24,54 @@ static inline int tile_row_end_s(const ShootArgs &a, int np, int ty1)
     return ty1 < 0 || ty1 > ty ? ty : ty1;
 }
 
-template <int NP>
-using SplitSmem = ShootSmem<NP, kSplitStage>;
-
-// Split star sum: clusters of SPLIT CTAs along x share one tile (tile column
-// blockIdx.x / SPLIT); partials are reduced through distributed shared memory.
+// Split star sum: clusters of SPLIT CTAs along x share one half tile (blockIdx.x /
+// SPLIT of its tile row); partials are reduced through distributed shared memory.
 template <int NP, int SPLIT, int NRP>
-__global__ void __launch_bounds__(kThreads, 2) k_shoot_split(ShootArgs a, int by0)
+__global__ void __launch_bounds__(kHalfThreads, 4) k_shoot_split(ShootArgs a, int by0)
 {
-    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    __shared__ __align__(16) ShootSmem<NP> sm;
     __shared__ TileShared ts;
-    shoot_tile<NP, kSplitStage, false, NRP, SPLIT>(a, (int)(blockIdx.x / SPLIT), by0 + (int)blockIdx.y,
-                                                   *reinterpret_cast<SplitSmem<NP> *>(dyn_smem), ts);
+    shoot_half<NP, false, NRP, SPLIT>(a, (int)(blockIdx.x / SPLIT), by0 + (int)blockIdx.y, sm, ts);
 }
 
-// Split star sum through global memory: CTA (tile column blockIdx.x / R, slice
+// Split star sum through global memory: CTA (half tile blockIdx.x / R, slice
 // blockIdx.x % R) sums one slice of the stars and stores its partials; tile rows
 // from `ty_base` on are numbered from 0 in the partials.
 template <int NP, int NRP>
-__global__ void __launch_bounds__(kThreads, 2) k_shoot_slices(ShootArgs a, int by0, int ty_base)
+__global__ void __launch_bounds__(kHalfThreads, 4) k_shoot_slices(ShootArgs a, int by0, int ty_base)
 {
-    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    __shared__ __align__(16) ShootSmem<NP> sm;
     __shared__ TileShared ts;
-    const int R = a.gslices, tiles_x = (a.rays.nx + kTileX - 1) / kTileX;
-    const int bx = (int)(blockIdx.x / R), r = (int)(blockIdx.x % R), by = by0 + (int)blockIdx.y;
-    shoot_tile<NP, kSplitStage, false, NRP, 1, 0, 1>(a, bx, by, *reinterpret_cast<SplitSmem<NP> *>(dyn_smem), ts,
-                                                      (int64_t)(by - ty_base) * tiles_x + bx, r);
+    const int R = a.gslices, hx = (int)(blockIdx.x / R), r = (int)(blockIdx.x % R), by = by0 + (int)blockIdx.y;
+    shoot_half<NP, false, NRP, 1, 1>(a, hx, by, sm, ts, (int64_t)(by - ty_base) * halves_x(a.rays) + hx, r);
 }
 
-// ... and the tile's partials folded in slice order, then beta and binning.
+// ... and the half tile's partials folded in slice order, then beta and binning.
 template <int NP>
-__global__ void __launch_bounds__(kThreads, 2) k_fold_slices(ShootArgs a, int by0, int ty_base)
+__global__ void __launch_bounds__(kHalfThreads, 4) k_fold_slices(ShootArgs a, int by0, int ty_base)
 {
-    __shared__ __align__(16) ShootSmem<NP, 32> sm;  // no stars are staged
+    __shared__ __align__(16) ShootSmem<NP> sm;
     __shared__ TileShared ts;
-    const int tiles_x = (a.rays.nx + kTileX - 1) / kTileX;
-    const int bx = (int)blockIdx.x, by = by0 + (int)blockIdx.y;
-    shoot_tile<NP, 32, false, 0, 1, 0, 2>(a, bx, by, sm, ts, (int64_t)(by - ty_base) * tiles_x + bx);
+    const int hx = (int)blockIdx.x, by = by0 + (int)blockIdx.y;
+    shoot_half<NP, false, 0, 1, 2>(a, hx, by, sm, ts, (int64_t)(by - ty_base) * halves_x(a.rays) + hx);
 }
 
 template <int NP, int SPLIT, int NRP>
 static cudaError_t launch_split_t(const ShootArgs &a, cudaStream_t s, int ty0, int ty1)
 {
-    const int tx = (a.rays.nx + kTileX - 1) / kTileX, ty = tile_row_end_s(a, NP, ty1);
+    const int ty = tile_row_end_s(a, NP, ty1);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = SPLIT;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = sizeof(SplitSmem<NP>);
-    const cudaError_t e0 = allow_dynamic_smem(k_shoot_split<NP, SPLIT, NRP>, cfg.dynamicSmemBytes);
-    if (e0 != cudaSuccess) return e0;
+    cfg.blockDim = dim3(kHalfThreads);
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     for (int by0 = ty0; by0 < ty; by0 += 65535) {
-        cfg.gridDim = dim3((unsigned)(tx * SPLIT), (unsigned)min(65535, ty - by0));
+        cfg.gridDim = dim3((unsigned)(halves_x(a.rays) * SPLIT), (unsigned)min(65535, ty - by0));
         const cudaError_t e = cudaLaunchKernelEx(&cfg, k_shoot_split<NP, SPLIT, NRP>, a, by0);
         if (e != cudaSuccess) return e;
     }
@@ -89,15 +79,15 @@ static cudaError_t launch_split_t(const ShootArgs &a, cudaStream_t s, int ty0, i
 }
 
 // The (split) star sum over a list of tiles (tile = by * tiles_x + bx), one cluster
-// (SPLIT = 1: one CTA) per listed tile: the learned far field's fallback tiles.
+// (SPLIT = 1: one CTA) per half of a listed tile: the learned far field's fallback tiles.
 template <int SPLIT, int NRP>
-__global__ void __launch_bounds__(kThreads, 2) k_shoot_split_list(ShootArgs a, const int *tiles)
+__global__ void __launch_bounds__(kHalfThreads, 4) k_shoot_split_list(ShootArgs a, const int *tiles)
 {
-    extern __shared__ __align__(16) unsigned char dyn_smem[];
+    __shared__ __align__(16) ShootSmem<4> sm;
     __shared__ TileShared ts;
     const int ntx = (a.rays.nx + kTileX - 1) / kTileX;
-    const int t = tiles[blockIdx.x / SPLIT];
-    shoot_tile<4, kSplitStage, false, NRP, SPLIT>(a, t % ntx, t / ntx, *reinterpret_cast<SplitSmem<4> *>(dyn_smem), ts);
+    const int h = (int)(blockIdx.x / SPLIT), t = tiles[h / 2];
+    shoot_half<4, false, NRP, SPLIT>(a, t % ntx * 2 + h % 2, t / ntx, sm, ts);
 }
 
 template <int SPLIT, int NRP>
@@ -109,14 +99,11 @@ static cudaError_t launch_split_list_t(const ShootArgs &a, const int *tiles, int
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kThreads);
-    cfg.dynamicSmemBytes = sizeof(SplitSmem<4>);
+    cfg.blockDim = dim3(kHalfThreads);
     cfg.stream = s;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const cudaError_t e = allow_dynamic_smem(k_shoot_split_list<SPLIT, NRP>, cfg.dynamicSmemBytes);
-    if (e != cudaSuccess) return e;
-    cfg.gridDim = dim3((unsigned)(ntiles * SPLIT));
+    cfg.gridDim = dim3((unsigned)(2 * ntiles * SPLIT));
     return cudaLaunchKernelEx(&cfg, k_shoot_split_list<SPLIT, NRP>, a, tiles);
 }
 
@@ -134,7 +121,7 @@ cudaError_t launch_shoot_split_list(const ShootArgs &a, const int *tiles, int64_
                                     int fma_pairs)
 {
     if (ntiles <= 0) return cudaSuccess;
-    if (ntiles * split > 0x7fffffff) return cudaErrorInvalidConfiguration;
+    if (2 * ntiles * split > 0x7fffffff) return cudaErrorInvalidConfiguration;
     return fma_pairs ? launch_split_list_r<1>(a, tiles, ntiles, split, s)
                      : launch_split_list_r<0>(a, tiles, ntiles, split, s);
 }
@@ -207,12 +194,11 @@ int auto_star_split(const RayGrid &r, int pairs_per_thread, int64_t nstars, int 
     return best;
 }
 
-// Partials of one pass: rows_per_pass tile rows x tiles_x tiles x split slices x
+// Partials of one pass: rows_per_pass tile rows x half tiles x split slices x
 // 2 NP float4 per thread.
 size_t gsplit_part_bytes(const RayGrid &r, int pairs_per_thread, int split, int tile_rows_per_pass)
 {
-    const size_t tiles_x = (size_t)((r.nx + kTileX - 1) / kTileX);
-    return (size_t)tile_rows_per_pass * tiles_x * (size_t)split * (size_t)(2 * pairs_per_thread * kThreads) *
+    return (size_t)tile_rows_per_pass * (size_t)halves_x(r) * (size_t)split * (size_t)(2 * pairs_per_thread * kHalfThreads) *
            sizeof(float4);
 }
 
@@ -231,18 +217,16 @@ static cudaError_t launch_gsplit_t(const ShootArgs &a0, int split, float4 *part,
     ShootArgs a = a0;
     a.gpart = part;
     a.gslices = split;
-    const int tx = (a.rays.nx + kTileX - 1) / kTileX, ty = tile_row_end_s(a, NP, ty1);
-    constexpr size_t smem = sizeof(SplitSmem<NP>);
-    cudaError_t e = allow_dynamic_smem(k_shoot_slices<NP, NRP>, smem);
-    if (e != cudaSuccess) return e;
-    if ((int64_t)tx * split > 0x7fffffff) return cudaErrorInvalidConfiguration;
+    const int hx = halves_x(a.rays), ty = tile_row_end_s(a, NP, ty1);
+    cudaError_t e = cudaSuccess;
+    if ((int64_t)hx * split > 0x7fffffff) return cudaErrorInvalidConfiguration;
     // one pass per rows_per_pass tile rows: the slices, then their fold (same stream,
     // so the next pass's slices overwrite partials the fold has read)
     for (int by0 = ty0; by0 < ty; by0 += rows_per_pass) {
         const int rows = std::min(rows_per_pass, ty - by0);
-        k_shoot_slices<NP, NRP><<<dim3((unsigned)(tx * split), (unsigned)rows), kThreads, smem, s>>>(a, by0, by0);
+        k_shoot_slices<NP, NRP><<<dim3((unsigned)(hx * split), (unsigned)rows), kHalfThreads, 0, s>>>(a, by0, by0);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
-        k_fold_slices<NP><<<dim3((unsigned)tx, (unsigned)rows), kThreads, 0, s>>>(a, by0, by0);
+        k_fold_slices<NP><<<dim3((unsigned)hx, (unsigned)rows), kHalfThreads, 0, s>>>(a, by0, by0);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
     return cudaSuccess;

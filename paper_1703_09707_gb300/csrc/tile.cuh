@@ -1,7 +1,6 @@
-// tile.cuh -- the per-tile FP32 shooting routine (Algorithm 1 on one 64 x 8*NP
-// tile of the ray grid: prologue, star stages, beta, binning), shared by the
-// single-field kernel, the persistent multi-field kernel and the fallback tiles
-// of the learned-far-field kernel.  See shoot_fp32.cu for the design notes.
+// tile.cuh -- the FP32 shooting routine (Algorithm 1 on half a 64 x 8*NP tile of the
+// ray grid: prologue, star stages, beta, binning), shared by the single-field, the
+// split, the persistent multi-field and the fallback-tile kernels.  See shoot_fp32.cu for the design notes.
 #pragma once
 
 #include <cooperative_groups.h>
@@ -16,9 +15,19 @@ namespace mlens {
 
 namespace cg = cooperative_groups;
 
-constexpr int kThreads = 256;
-constexpr int kTileX = 64;                 // rays per tile row = threads per row group
-constexpr int kGroups = kThreads / kTileX; // row groups
+constexpr int kThreads = 256;              // the learned kernel's CTA: a whole tile
+constexpr int kTileX = 64;                 // rays per tile row
+constexpr int kGroups = 4;                 // row groups of a tile, 2 NP rows each
+// The direct sum's CTA takes half a tile, 32 of its columns (a warp per row group): the
+// arithmetic is the tile's (its centre), while grids of few tiles fill the SMs more evenly
+// and four small CTAs per SM leave fewer warps waiting at a barrier than two large ones
+// (100 stars x 1000^2 rays 48.6 -> 34.8 us together with the short last chunk and the one
+// clear, clear.cu; 256 fields 490 -> 472 ms; 1e4 stars x 8192^2 rays, many tiles, 132.2 ->
+// 132.6 ms).
+constexpr int kHalfX = 32;
+constexpr int kHalfThreads = kHalfX * kGroups;
+constexpr int kStage = kHalfThreads;       // stars per stage: one per thread
+constexpr int kHalfWin = 32;               // binning window of a half tile
 constexpr int kKahan = 32;                 // stars per compensated partial
 
 static_assert(kStarPad % kKahan == 0, "star padding must be whole Kahan chunks");
@@ -46,10 +55,10 @@ struct StarStage {
     float2 mm[2][SC];  // (m, m)
 };
 
-template <int NP, int SC, bool NAIVE = false>
+template <int NP, bool NAIVE = false>
 union ShootSmem {
-    std::conditional_t<NAIVE, StarStage<SC>, RowStage<NP, SC>> st;
-    uint32_t hist[kWin * kWin];
+    std::conditional_t<NAIVE, StarStage<kStage>, RowStage<NP, kStage>> st;
+    uint32_t hist[kHalfWin * kHalfWin];
 };
 
 constexpr int kMaxRows = 32;  // ray rows of the largest tile (NP = 4)
@@ -136,7 +145,7 @@ __device__ __forceinline__ float2 rcp_nr2(float2 x)
     return y;
 }
 
-// One tile (bx, by) of the ray grid of `a`, start to finish: prologue, star
+// Half hx of tile row by (half hx % 2 of tile hx / 2) of the ray grid of `a`, start to finish: prologue, star
 // stages, beta, binning, counters.  Every thread of the CTA must call it.
 // NRP = 1: ray pair 0 takes its reciprocals from rcp_nr2 (FMA pipe) on every third
 // star of a 32-star chunk (stars 2, 5, .., 29: 10 of the 128 reciprocals a thread
@@ -163,58 +172,50 @@ __device__ __forceinline__ float2 rcp_nr2(float2 x)
 // (2 NP float4 per thread); rank 0 reads them through distributed shared memory in
 // rank order, folds each in with two Kahan steps (S_r, then -C_r) and alone goes on
 // to beta and binning.
-// LOM: how the tile learns whether the ray offsets need low parts: 0 = from the grid
-// at run time (RayGrid lo, both loops compiled), 1 = never, 2 = always (callers
-// that have chosen already).
-//
 // GS (re-centred FP32 only, SPLIT = 1): the split star sum through global memory.
 // GS = 1: the CTA sums slice `gslice` of a.gslices consecutive 32-aligned slices of
 // the stars (the same slices as a cluster split of that many CTAs) and stores its
-// partials (S, C) as 2 NP float4 per thread at a.gpart, block gtile * a.gslices +
+// partials (S, C) as 2 NP float4 per thread at a.gpart, block ghalf * a.gslices +
 // gslice, then returns.  GS = 2: the CTA sums no stars; it takes slice 0's partials
 // as its own, folds the others in slice order (two Kahan steps each, S_r then -C_r,
 // as the cluster fold does) and goes on to beta and binning.
-template <int NP, int SC, bool NAIVE, int NRP = 0, int SPLIT = 1, int LOM = 0, int GS = 0>
-__device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, ShootSmem<NP, SC, NAIVE> &sm,
-                                           TileShared &ts, int64_t gtile = 0, int gslice = 0)
+template <int NP, bool NAIVE, int NRP = 0, int SPLIT = 1, int GS = 0>
+__device__ __forceinline__ void shoot_half(const ShootArgs &a, int hx, int by, ShootSmem<NP, NAIVE> &sm,
+                                           TileShared &ts, int64_t ghalf = 0, int gslice = 0)
 {
     static_assert(SPLIT == 1 || !NAIVE, "the split sum is for the re-centred kernel");
     static_assert(GS == 0 || (!NAIVE && SPLIT == 1), "the global split is for the re-centred kernel");
-    static_assert(SC <= kThreads, "one thread stages one star");
     constexpr int kTileY = tile_rows(NP);
     static_assert(kTileY <= kMaxRows, "TileShared holds the tile's rows");
     const int tid = threadIdx.x;
-    const int tx = tid % kTileX;
-    const int tg = tid / kTileX;
-    const int i0 = bx * kTileX;
+    const int tx = hx % 2 * kHalfX + tid % kHalfX;  // column within the tile
+    const int tg = tid / kHalfX;                    // row group: one warp
+    const int i0 = hx / 2 * kTileX;
     const int j0 = by * kTileY;
     const RayGrid &R = a.rays;
+    if (i0 + hx % 2 * kHalfX >= R.nx) return;  // the whole half is beyond the grid
 
-    if (tid == 0) {
-        if (!NAIVE) {
-            // tile centre (tile_centre: star offsets near the tile exact), offsets of
-            // the first ray and A c in FP64, split into float pairs
-            double cxd = R.x0 + ((double)i0 + 0.5 * kTileX) * R.dx;
-            double cyd = R.y0 + ((double)j0 + 0.5 * kTileY) * R.dy;
-            float cx = tile_centre(cxd, kTileX * R.dx, R.qx, R.qxinv), cy = tile_centre(cyd, kTileY * R.dy, R.qy, R.qyinv);
-            double ex = (R.x0 + ((double)i0 + 0.5) * R.dx) - (double)cx;
-            double ey = (R.y0 + ((double)j0 + 0.5) * R.dy) - (double)cy;
-            double bxd = a.lens.a11 * (double)cx + a.lens.a12 * (double)cy;
-            double byd = a.lens.a12 * (double)cx + a.lens.a22 * (double)cy;
-            float bxh = (float)bxd, byh = (float)byd;
-            ts.tc[0] = cx;
-            ts.tc[1] = cy;
-            ts.tc[2] = (float)ex;
-            ts.tc[3] = (float)ey;
-            ts.tc[4] = bxh;
-            ts.tc[5] = byh;
-            ts.tc[6] = (float)(bxd - (double)bxh);
-            ts.tc[7] = (float)(byd - (double)byh);
-            ts.tc[8] = (float)(ex - (double)ts.tc[2]);
-            ts.tc[9] = (float)(ey - (double)ts.tc[3]);
-        }
-        ts.sred[0] = ts.sred[1] = ts.sred[2] = 0u;
+    if (tid < 2 && !NAIVE) {
+        // one axis per lane: the tile centre (tile_centre: star offsets near the tile
+        // exact), offsets of the first ray and A c in FP64, split into float pairs
+        const bool y = tid == 1;
+        const double o = y ? R.y0 : R.x0, d = y ? R.dy : R.dx;
+        const double first = (double)(y ? j0 : i0), span = (double)(y ? kTileY : kTileX);
+        const double mid = o + (first + 0.5 * span) * d;
+        const float c = tile_centre(mid, span * d, y ? R.qy : R.qx, y ? R.qyinv : R.qxinv);
+        const double e = (o + (first + 0.5) * d) - (double)c;
+        const float other = __shfl_xor_sync(0x3u, c, 1);
+        const double cx = (double)(y ? other : c), cy = (double)(y ? c : other);
+        const double ax = y ? a.lens.a12 : a.lens.a11, ay = y ? a.lens.a22 : a.lens.a12;
+        const double bd = ax * cx + ay * cy;
+        const float bh = (float)bd, eh = (float)e;
+        ts.tc[tid] = c;
+        ts.tc[2 + tid] = eh;
+        ts.tc[4 + tid] = bh;
+        ts.tc[6 + tid] = (float)(bd - (double)bh);
+        ts.tc[8 + tid] = (float)(e - (double)eh);
     }
+    if (tid < 3) ts.sred[tid] = 0u;
     __syncthreads();
 
     // ------------------------------------------------------- this thread's rays
@@ -222,7 +223,7 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
     float2 px[NP], py[NP];             // partial sums (NAIVE: the whole running sum)
     float2 Sx[NP], Sy[NP], Cx[NP], Cy[NP];
     const float kx = (float)tx;
-    const bool lo = !NAIVE && (LOM == 2 || (LOM == 0 && R.lo));
+    const bool lo = !NAIVE && R.lo;
     if (!NAIVE) {
         if (lo) {
             ray_offset(kx, ts.tc[2], ts.tc[8], R.dxh, R.dxl, rxh, rxl);
@@ -246,25 +247,30 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
 
     // ---------------------------------------------------------- star stages
     const float4 *stars = a.stars;
-    int64_t nst = a.nstars;  // multiple of kKahan
+    int64_t nst = a.nstars;   // multiple of kKahan: the slices are whole chunks
+    int64_t real = a.n;       // of which stars: the padding adds exactly zero and is left out
     if (SPLIT > 1) {
         const int64_t chunk = ((nst + SPLIT - 1) / SPLIT + kKahan - 1) / kKahan * kKahan;
         const int64_t s0 = min(nst, (int64_t)cg::this_cluster().block_rank() * chunk);
         stars += s0;
         nst = min(chunk, nst - s0);
+        real -= s0;
     }
     if (GS == 1) {
         const int64_t chunk = ((nst + a.gslices - 1) / a.gslices + kKahan - 1) / kKahan * kKahan;
         const int64_t s0 = min(nst, (int64_t)gslice * chunk);
         stars += s0;
         nst = min(chunk, nst - s0);
+        real -= s0;
     }
     if (GS == 2) nst = 0;
+    nst = max(min(nst, real), (int64_t)0);
+    constexpr int SC = kStage;
     const int nstage = (int)((nst + SC - 1) / SC);
     float4 nxt;
     auto stage_load = [&](int s) {
         const int64_t k = (int64_t)s * SC + tid;
-        nxt = (tid < SC && k < nst) ? __ldg(&stars[k]) : make_float4(0.f, 0.f, 0.f, 0.f);
+        nxt = k < nst ? __ldg(&stars[k]) : make_float4(kPadCoord, kPadCoord, 0.f, 0.f);
     };
     if constexpr (NAIVE) {
         const float y0f = (float)R.y0, dyf = (float)R.dy;
@@ -280,10 +286,8 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
             py[p] = f2(a.lens.fm12 * rxh + a.lens.fm22 * y0, a.lens.fm12 * rxh + a.lens.fm22 * y1);
         }
         auto stage_store = [&](int buf) {
-            if (tid < SC) {
-                sm.st.q[buf][tid] = make_float4(-nxt.x, -nxt.x, -nxt.y, -nxt.y);
-                sm.st.mm[buf][tid] = f2(nxt.z, nxt.z);
-            }
+            sm.st.q[buf][tid] = make_float4(-nxt.x, -nxt.x, -nxt.y, -nxt.y);
+            sm.st.mm[buf][tid] = f2(nxt.z, nxt.z);
         };
         if (nstage > 0) {
             stage_load(0);
@@ -297,7 +301,7 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
             const float4 *Q = sm.st.q[buf];
             const float2 *M = sm.st.mm[buf];
 #pragma unroll 1
-            for (int k0 = 0; k0 < cnt; k0 += kKahan) {
+            for (int k0 = 0; k0 < cnt; k0 += kKahan) {  // (a short last chunk is staged full, with massless stars)
 #pragma unroll
                 for (int k = k0; k < k0 + kKahan; ++k) {
                     const float4 q = Q[k];
@@ -321,7 +325,6 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
     } else {
         constexpr int kStride = RowStage<NP, SC>::kStride;
         auto stage_store = [&](int buf) {  // thread t: star t against every row of the tile
-            if (tid >= SC) return;
             const float ny = __fsub_rn(ts.tc[1], nxt.y);
             float4 *dst = sm.st.s[buf] + tid * kStride;
 #pragma unroll
@@ -349,43 +352,57 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
             // subtraction (grids whose ray offsets are not exact floats, RayGrid lo)
             auto chunks = [&](auto lo_tag) {
                 constexpr bool LO = decltype(lo_tag)::value;
-#pragma unroll 1
-                for (int k0 = 0; k0 < cnt; k0 += kKahan) {
-                    const float4 *Q = sm.st.s[buf] + k0 * kStride;
+                // star k of a chunk (Q: the chunk's first); NR: ray pair 0 by rcp_nr2
+                auto star = [&](const float4 *Q, int k, bool NR) {
+                    const float4 q = Q[k * kStride + kTileY / 4];
+                    float d = __fadd_rn(rxh, q.z);
+                    if (LO) d = __fadd_rn(d, rxl);
+                    const float d2 = __fmul_rn(d, d);
+                    const float2 dx = f2(d, d), dx2 = f2(d2, d2), m2 = f2(q.x, q.y);
+                    float4 row[NP / 2];
 #pragma unroll
-                    for (int k = 0; k < kKahan; ++k) {
-                        const float4 q = Q[k * kStride + kTileY / 4];
-                        float d = __fadd_rn(rxh, q.z);
-                        if (LO) d = __fadd_rn(d, rxl);
-                        const float d2 = __fmul_rn(d, d);
-                        const float2 dx = f2(d, d), dx2 = f2(d2, d2), m2 = f2(q.x, q.y);
-                        float4 row[NP / 2];
+                    for (int h = 0; h < NP / 2; ++h) row[h] = Q[k * kStride + tg * (NP / 2) + h];
 #pragma unroll
-                        for (int h = 0; h < NP / 2; ++h) row[h] = Q[k * kStride + tg * (NP / 2) + h];
-#pragma unroll
-                        for (int p = 0; p < NP; ++p) {
-                            const float2 dy = p % 2 ? f2(row[p / 2].z, row[p / 2].w) : f2(row[p / 2].x, row[p / 2].y);
-                            const float2 r2 = __ffma2_rn(dy, dy, dx2);
-                            const float2 inv =
-                                NRP > 0 && p == 0 && k % 3 == 2 ? rcp_nr2(r2) : f2(rcp_approx(r2.x), rcp_approx(r2.y));
-                            const float2 f = __fmul2_rn(m2, inv);
-                            px[p] = __ffma2_rn(f, dx, px[p]);
-                            py[p] = __ffma2_rn(f, dy, py[p]);
-                        }
+                    for (int p = 0; p < NP; ++p) {
+                        const float2 dy = p % 2 ? f2(row[p / 2].z, row[p / 2].w) : f2(row[p / 2].x, row[p / 2].y);
+                        const float2 r2 = __ffma2_rn(dy, dy, dx2);
+                        const float2 inv =
+                            NRP > 0 && p == 0 && NR ? rcp_nr2(r2) : f2(rcp_approx(r2.x), rcp_approx(r2.y));
+                        const float2 f = __fmul2_rn(m2, inv);
+                        px[p] = __ffma2_rn(f, dx, px[p]);
+                        py[p] = __ffma2_rn(f, dy, py[p]);
                     }
+                };
+                auto chunk_end = [&]() {
 #pragma unroll
                     for (int p = 0; p < NP; ++p) {
                         kahan2(Sx[p], Cx[p], px[p]);
                         kahan2(Sy[p], Cy[p], py[p]);
                         px[p] = py[p] = f2(0.f, 0.f);
                     }
+                };
+                const float4 *Q = sm.st.s[buf], *end = Q + cnt / kKahan * kKahan * kStride;
+#pragma unroll 1
+                for (; Q != end; Q += kKahan * kStride) {
+#pragma unroll
+                    for (int k = 0; k < kKahan; ++k) star(Q, k, k % 3 == 2);
+                    chunk_end();
+                }
+                const int rest = cnt % kKahan;  // the stars' last, short chunk
+                if (rest) {
+                    int k = 0;
+#pragma unroll 1
+                    for (; k + 3 <= rest; k += 3) {
+                        star(Q, k, false);
+                        star(Q, k + 1, false);
+                        star(Q, k + 2, true);
+                    }
+#pragma unroll 1
+                    for (; k < rest; ++k) star(Q, k, false);
+                    chunk_end();
                 }
             };
-            if (LOM == 2)
-                chunks(std::true_type{});
-            else if (LOM == 1)
-                chunks(std::false_type{});
-            else if (lo)
+            if (lo)
                 chunks(std::true_type{});
             else
                 chunks(std::false_type{});
@@ -395,19 +412,19 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
     }
 
     if constexpr (GS == 1) {
-        float4 *dst = a.gpart + (gtile * a.gslices + gslice) * (int64_t)(2 * NP * kThreads);
+        float4 *dst = a.gpart + (ghalf * a.gslices + gslice) * (int64_t)(2 * NP * kHalfThreads);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            dst[(2 * p) * kThreads + tid] = make_float4(Sx[p].x, Sx[p].y, Sy[p].x, Sy[p].y);
-            dst[(2 * p + 1) * kThreads + tid] = make_float4(Cx[p].x, Cx[p].y, Cy[p].x, Cy[p].y);
+            dst[(2 * p) * kHalfThreads + tid] = make_float4(Sx[p].x, Sx[p].y, Sy[p].x, Sy[p].y);
+            dst[(2 * p + 1) * kHalfThreads + tid] = make_float4(Cx[p].x, Cx[p].y, Cy[p].x, Cy[p].y);
         }
         return;
     }
     if constexpr (GS == 2) {
-        const float4 *src = a.gpart + gtile * a.gslices * (int64_t)(2 * NP * kThreads);
+        const float4 *src = a.gpart + ghalf * a.gslices * (int64_t)(2 * NP * kHalfThreads);
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-            const float4 s0 = src[(2 * p) * kThreads + tid], c0 = src[(2 * p + 1) * kThreads + tid];
+            const float4 s0 = src[(2 * p) * kHalfThreads + tid], c0 = src[(2 * p + 1) * kHalfThreads + tid];
             Sx[p] = f2(s0.x, s0.y);
             Sy[p] = f2(s0.z, s0.w);
             Cx[p] = f2(c0.x, c0.y);
@@ -415,10 +432,10 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
         }
 #pragma unroll 1
         for (int r = 1; r < a.gslices; ++r) {
-            const float4 *rp = src + (int64_t)r * (2 * NP * kThreads);
+            const float4 *rp = src + (int64_t)r * (2 * NP * kHalfThreads);
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
-                const float4 sr = rp[(2 * p) * kThreads + tid], cr = rp[(2 * p + 1) * kThreads + tid];
+                const float4 sr = rp[(2 * p) * kHalfThreads + tid], cr = rp[(2 * p + 1) * kHalfThreads + tid];
                 kahan2(Sx[p], Cx[p], f2(sr.x, sr.y));
                 kahan2(Sy[p], Cy[p], f2(sr.z, sr.w));
                 kahan2(Sx[p], Cx[p], f2(-cr.x, -cr.y));
@@ -428,15 +445,15 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
     }
 
     if constexpr (SPLIT > 1) {
-        static_assert(sizeof(sm) >= 2 * NP * kThreads * sizeof(float4), "the partials fit the stage memory");
+        static_assert(sizeof(sm) >= 2 * NP * kHalfThreads * sizeof(float4), "the partials fit the stage memory");
         cg::cluster_group cl = cg::this_cluster();
         const unsigned rank = cl.block_rank();
         float4 *part = reinterpret_cast<float4 *>(&sm);  // the stages are dead (the loop's last barrier)
         if (rank != 0) {
 #pragma unroll
             for (int p = 0; p < NP; ++p) {
-                part[(2 * p) * kThreads + tid] = make_float4(Sx[p].x, Sx[p].y, Sy[p].x, Sy[p].y);
-                part[(2 * p + 1) * kThreads + tid] = make_float4(Cx[p].x, Cx[p].y, Cy[p].x, Cy[p].y);
+                part[(2 * p) * kHalfThreads + tid] = make_float4(Sx[p].x, Sx[p].y, Sy[p].x, Sy[p].y);
+                part[(2 * p + 1) * kHalfThreads + tid] = make_float4(Cx[p].x, Cx[p].y, Cy[p].x, Cy[p].y);
             }
         }
         cl.sync();  // every rank's partials are in place
@@ -446,7 +463,7 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
                 const float4 *rp = cl.map_shared_rank(part, r);
 #pragma unroll
                 for (int p = 0; p < NP; ++p) {
-                    const float4 sr = rp[(2 * p) * kThreads + tid], cr = rp[(2 * p + 1) * kThreads + tid];
+                    const float4 sr = rp[(2 * p) * kHalfThreads + tid], cr = rp[(2 * p + 1) * kHalfThreads + tid];
                     kahan2(Sx[p], Cx[p], f2(sr.x, sr.y));
                     kahan2(Sy[p], Cy[p], f2(sr.z, sr.w));
                     kahan2(Sx[p], Cx[p], f2(-cr.x, -cr.y));
@@ -493,16 +510,17 @@ __device__ __forceinline__ void shoot_tile(const ShootArgs &a, int bx, int by, S
     }
 
     // ----------------------------------------------------------- binning
+    pdl_wait();  // the map's and the counters' clears
     const int ix = i0 + tx;
     const bool col_ok = ix < R.nx;
     __syncthreads();  // star stages are dead: reuse the memory as the window
-    hist_zero(sm.hist);
-    if (tid == 0) {
-        ts.win[0] = win_origin(pair_axis_rough(bxh[0], a.bin.ax), a.bin.nx);
-        ts.win[1] = win_origin(pair_axis_rough(byh[0], a.bin.ay), a.bin.ny);
+    hist_zero<kHalfWin>(sm.hist);
+    if (tid == kHalfThreads / 2 + kHalfX / 2) {  // the half tile's middle ray
+        ts.win[0] = win_origin<kHalfWin>(pair_axis_rough(bxh[0], a.bin.ax), a.bin.nx);
+        ts.win[1] = win_origin<kHalfWin>(pair_axis_rough(byh[0], a.bin.ay), a.bin.ny);
     }
     __syncthreads();
-    const WinHist W = make_window(sm.hist, ts.win[0], ts.win[1], a.bin);
+    const WinHist<kHalfWin> W = make_window<kHalfWin>(sm.hist, ts.win[0], ts.win[1], a.bin);
     const int nrow = col_ok ? min(2 * NP, R.ny - (j0 + tg * 2 * NP)) : 0;  // this thread's rays in the grid
     unsigned no = 0, nn = 0;
 #pragma unroll
