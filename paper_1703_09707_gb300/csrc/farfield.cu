@@ -1213,6 +1213,84 @@ cudaError_t ff_flags(const unsigned *maxerr, int nrc, float tol, int *flags, cud
 }
 
 // ================================================ learned shooting kernel
+// What the tiles of a learned map need beyond the stars, laid out once per fit: per tile
+// its centre, offsets and A c (FP64 work), its near stars' CSR runs and its place in its
+// cell; per cell the series as the kernel's packed arithmetic takes it, and e_c / 2.  Formed
+// by one thread at each tile's start, the same values cost the series-only map a fifth of
+// its time: a chain of FP64 instructions and dependent loads while the CTA waited.
+__global__ void k_tile_desc(const int *tiles, int64_t n, RayGrid R, LensTerms lens, CellGrid cg, const int *cstart,
+                            TileDesc *out)
+{
+    const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    constexpr int kTileY = 32;
+    const int ntx = (R.nx + kTileX - 1) / kTileX, tile = tiles[k];
+    const int bx = tile % ntx, by = tile / ntx, i0 = bx * kTileX, j0 = by * kTileY;
+    TileDesc d{};
+    const double cxd = R.x0 + ((double)i0 + 0.5 * kTileX) * R.dx;
+    const double cyd = R.y0 + ((double)j0 + 0.5 * kTileY) * R.dy;
+    const float fcx = tile_centre(cxd, kTileX * R.dx, R.qx, R.qxinv);
+    const float fcy = tile_centre(cyd, kTileY * R.dy, R.qy, R.qyinv);
+    const double ex = (R.x0 + ((double)i0 + 0.5) * R.dx) - (double)fcx;
+    const double ey = (R.y0 + ((double)j0 + 0.5) * R.dy) - (double)fcy;
+    const double bxd = lens.a11 * (double)fcx + lens.a12 * (double)fcy;
+    const double byd = lens.a12 * (double)fcx + lens.a22 * (double)fcy;
+    const float bxh = (float)bxd, byh = (float)byd;
+    d.tc[0] = fcx;
+    d.tc[1] = fcy;
+    d.tc[2] = (float)ex;
+    d.tc[3] = (float)ey;
+    d.tc[4] = bxh;
+    d.tc[5] = byh;
+    d.tc[6] = (float)(bxd - (double)bxh);
+    d.tc[7] = (float)(byd - (double)byh);
+    d.tc[8] = (float)(ex - (double)d.tc[2]);
+    d.tc[9] = (float)(ey - (double)d.tc[3]);
+    const int cx = bx / cg.ktx, cy = by / cg.kty;
+    for (int q = 0; q < 3; ++q) {  // the 3 x 3 block's rows of cells (the ray cell is (cx + 1, cy + 1))
+        const int c = (cy + q) * cg.nx + cx;
+        d.near_at[q] = cstart[c];
+        d.near_n[q] = cstart[c + 3] - cstart[c];
+    }
+    d.bx = bx;
+    d.by = by;
+    d.rc = cy * cg.ncx + cx;
+    d.ioff = (bx % cg.ktx) * kTileX;
+    d.joff = (by % cg.kty) * kTileY;
+    out[k] = d;
+}
+
+cudaError_t ff_tile_desc(const int *tiles, int64_t n, const RayGrid &rays, const LensTerms &lens, const CellGrid &cg,
+                         const int *cstart, TileDesc *out, cudaStream_t s)
+{
+    if (n <= 0) return cudaSuccess;
+    k_tile_desc<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(tiles, n, rays, lens, cg, cstart, out);
+    return cudaGetLastError();
+}
+
+__global__ void k_cell_rec(const float *coef, const float *sc, const float *ec, int nrc, CellRec *out)
+{
+    const int rc = blockIdx.x, t = threadIdx.x;
+    const float *c = coef + (int64_t)rc * kCoefStride;
+    CellRec &o = out[rc];
+    if (t == 0) {
+        o.b0 = make_float4(c[0], c[1], c[2], c[3]);
+        o.sc = make_float4(sc[rc], 0.0f, 0.0f, 0.0f);
+    }
+    if (t < kPeMax) o.b[t] = make_float4(c[4 + 2 * t], c[4 + 2 * t], c[5 + 2 * t], c[5 + 2 * t]);
+    if (t < kNetPairs) {
+        const float *e = ec + (int64_t)rc * kHid + 2 * t;
+        o.ec[t] = make_float2(0.5f * e[0], 0.5f * e[1]);  // (exact)
+    }
+}
+
+cudaError_t ff_cell_rec(const float *coef, const float *sc, const float *ec, int nrc, CellRec *out, cudaStream_t s)
+{
+    k_cell_rec<<<(unsigned)nrc, 32, 0, s>>>(coef, sc, ec, nrc, out);
+    return cudaGetLastError();
+}
+
+constexpr int kLearnWin = 32;  // a learned tile's rays land on a patch of about 12 x 6 pixels
 struct LearnSmem {
     __align__(128) unsigned char w2cm[kHid * kHid * 2];  // W2 / 2 [out][in], BF16, core-matrix layout (B operand)
     uint64_t mbar[2];     // per warpgroup: completion of its tensor-core MMAs
@@ -1221,17 +1299,15 @@ struct LearnSmem {
     int wg_ok[8];         // per warp: the last wait completed
     int tc_dead[2];       // per warpgroup: a wait gave up; no more MMAs
     uint32_t pending[2];  // the phase a dead warpgroup still waits for
-    // the tile's cell embedding per pair of hidden units (c, c + 1), halved (the block
-    // forms v / 2, SiLU's argument); the shared constants come with the launch (NetConsts)
-    float2 ec2[kHid / 2];  // {e_c, e_c+1} / 2
-    float coef[kCoefStride];
-    float4 coef2[kPeMax];  // b_q as {Re, Re, Im, Im}: both rays of a pair at once
-    float sc;
-    int rb[3], re[3];
-    int nnear;
+    // the tile's cell: series and embedding (the constants the cells share come with the
+    // launch, NetConsts)
+    __align__(16) CellRec cell;
+    __align__(16) TileDesc desc[2];  // this tile's and the next one's
+    __align__(16) uint32_t hist[kLearnWin * kLearnWin];  // binning window, cleared as it is flushed
+    int win[2];
+    unsigned sred[3];
+    long long first;
 };
-
-__device__ __forceinline__ float2 cmul(float2 a, float2 b) { return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); }
 
 // SiLU of two hidden units at once, as silu_hw, from h = v / 2: h + h tanh(h) with
 // the hardware tanh (one packed FMA).  The learned kernel forms h directly: every
@@ -1243,149 +1319,154 @@ __device__ __forceinline__ float2 silu_half2(float2 h)
     return __ffma2_rn(h, make_float2(tanh_hw(h.x), tanh_hw(h.y)), h);
 }
 
-// One tile of a non-flagged cell: near stars exactly (FP32 recentred + Kahan,
-// as the plain kernel), far field = float-pair b0 + series to order pe +
-// network residual, then beta and the same binning epilogue.
-// Near-field stars per compensated chunk (a tile's 3 x 3 block holds ~1.3 stars per
-// ray at the learned workload's density; a chunk is padded with massless far stars):
-// 4 with the network, 2 for the series alone (measured fastest for each).
+// Near-field stars per compensated chunk (a tile's 3 x 3 block holds ~1.3 stars at the
+// learned workload's density): 4 with the network, 2 for the series alone.
 template <bool NET>
 constexpr int kNearChunk = NET ? 4 : 2;
 constexpr int kTcChunk = 128;                            // rays per tensor-core MMA (M)
 constexpr int kTcABytes = kTcChunk * kHid * 2;           // one warpgroup's A operand (16 KB)
 constexpr int kTcSmem = 2 * kTcABytes;                   // the two A operands
-union LearnTileSmem {  // the near-field star stage, then the window
-    StarStage<256> st;
-    uint32_t hist[kWin * kWin];
-};
-constexpr size_t kLearnedDynSmem = kTcSmem > sizeof(LearnTileSmem) ? kTcSmem : sizeof(LearnTileSmem);
+using NearStage = StarStage<256>;
+constexpr size_t kLearnedDynSmem = kTcSmem > sizeof(NearStage) ? kTcSmem : sizeof(NearStage);
+static_assert(sizeof(CellRec) % 16 == 0 && sizeof(CellRec) / 16 <= 64, "a cell record is copied by two warps");
+static_assert(sizeof(TileDesc) % 4 == 0 && sizeof(TileDesc) / 4 <= 32, "a descriptor is copied by one warp");
 
+__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
+{
+    const unsigned a = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(a), "l"(gmem) : "memory");
+}
+
+// The learned tiles: near stars exactly (FP32 re-centred + Kahan, as the plain kernel), far
+// field = float-pair b0 + series to order pe + network residual, then beta and binning, by
+// persistent CTAs that pull tiles from a queue.  While a tile is worked on, the queue is
+// asked for the next one and its descriptor fetched; the cell's record arrives by
+// asynchronous copies behind the near field; the window is cleared by the threads that flush
+// it; the ray counters stay in registers until the kernel ends.
+// NET: the network on the tensor cores (tcgen05; 128 tensor-memory columns and the
+// two A operands in dynamic shared memory, in the same bytes as the near stage);
+// without it (the series alone) the kernel carries no tensor-core code.
 // LO: the ray offsets carry low parts (grids whose offsets are not exact floats,
 // RayGrid lo); a separate instance so that the exact-offset tiles keep their
 // registers.
+// Four CTAs per SM (64 registers, spills included; tensor memory holds four CTAs' 128
+// columns): eight warps per scheduler hide the latency of the 128 hardware tanh per ray.
+// Three CTAs: 42.9 and 1.95 ms for the two maps below.
+// Bound with the network by MUFU (132 results a ray; 72 % busy), without it by issue slots.
+// 32768 x 33024 rays of 1e6 stars, no cell flagged: 44.3 -> 41.1 ms; 2.7e8 rays, order-16
+// series alone, 2.47 -> 1.92 ms: descriptors and records from the fit, the next tile
+// fetched ahead, one window clear and four barriers less a tile, near stars without
+// padding, two ray pairs per Horner step (one 2.13, four 1.97 ms).
 template <bool NET, bool LO>
-__device__ __forceinline__ void learned_tile(const LearnedArgs &L, int bx, int by, LearnTileSmem &sm, TileShared &ts,
-                                             LearnSmem &ls, unsigned char *abuf_all, uint32_t &phase)
+__global__ void __launch_bounds__(kThreads, 4) k_shoot_learned(const __grid_constant__ LearnedArgs L)
 {
     constexpr int NP = 4;
-    constexpr int kTileY = 32;
+    __shared__ __align__(128) LearnSmem ls;
+    extern __shared__ __align__(128) unsigned char dyn_smem[];
+    NearStage &near_st = *reinterpret_cast<NearStage *>(dyn_smem);
     const ShootArgs &a = L.plain;
     const RayGrid &R = a.rays;
-    const CellGrid &cg = L.cg;
     const int tid = threadIdx.x, tx = tid % kTileX, tg = tid / kTileX;
-    const int i0 = bx * kTileX, j0 = by * kTileY;
-    const int cx = bx / cg.ktx, cy = by / cg.kty, rc = cy * cg.ncx + cx;
-    if (tid == 0) {
-        double cxd = R.x0 + ((double)i0 + 0.5 * kTileX) * R.dx;
-        double cyd = R.y0 + ((double)j0 + 0.5 * kTileY) * R.dy;
-        float fcx = tile_centre(cxd, kTileX * R.dx, R.qx, R.qxinv);
-        float fcy = tile_centre(cyd, kTileY * R.dy, R.qy, R.qyinv);
-        double ex = (R.x0 + ((double)i0 + 0.5) * R.dx) - (double)fcx;
-        double ey = (R.y0 + ((double)j0 + 0.5) * R.dy) - (double)fcy;
-        double bxd = a.lens.a11 * (double)fcx + a.lens.a12 * (double)fcy;
-        double byd = a.lens.a12 * (double)fcx + a.lens.a22 * (double)fcy;
-        float bxh = (float)bxd, byh = (float)byd;
-        ts.tc[0] = fcx;
-        ts.tc[1] = fcy;
-        ts.tc[2] = (float)ex;
-        ts.tc[3] = (float)ey;
-        ts.tc[4] = bxh;
-        ts.tc[5] = byh;
-        ts.tc[6] = (float)(bxd - (double)bxh);
-        ts.tc[7] = (float)(byd - (double)byh);
-        ts.tc[8] = (float)(ex - (double)ts.tc[2]);
-        ts.tc[9] = (float)(ey - (double)ts.tc[3]);
-        ts.sred[0] = ts.sred[1] = ts.sred[2] = 0u;
-        const int ecx = cx + 1, ecy = cy + 1;
-        int tot = 0;
-        for (int d = -1; d <= 1; ++d) {
-            const int row = (ecy + d) * cg.nx;
-            ls.rb[d + 1] = L.cstart[row + ecx - 1];
-            ls.re[d + 1] = L.cstart[row + ecx + 2];
-            tot += ls.re[d + 1] - ls.rb[d + 1];
+    uint32_t phase = 0;  // completed MMA batches of this thread's warpgroup, mod 2
+    if (NET) {
+        for (int i = tid; i < kHid * kHid; i += kThreads)
+            *reinterpret_cast<__nv_bfloat16 *>(ls.w2cm + umma::cm_offset(i / kHid, i % kHid)) =
+                __float2bfloat16_rn(0.5f * __bfloat162float(L.w2b[i]));  // W2 / 2 (exact)
+        if (tid < 2) ls.tc_dead[tid] = 0;
+        if (tid == 0) {
+            umma::mbar_init(&ls.mbar[0], 1);
+            umma::mbar_init(&ls.mbar[1], 1);
+            umma::mbar_init(&ls.idle, 1);
+            umma::fence_mbar_init();
         }
-        ls.nnear = tot;
-        ls.sc = L.sc[rc];
+        if (tid < 32) umma::tmem_alloc(&ls.tmem, 2 * kHid);
+        umma::fence_async_smem();  // W2 is read by the tensor cores
+        umma::fence_before();
     }
-    if (tid < kCoefStride) ls.coef[tid] = L.coef[(int64_t)rc * kCoefStride + tid];
-    if (tid < kPeMax) {
-        const float re = L.coef[(int64_t)rc * kCoefStride + 4 + 2 * tid];
-        const float im = L.coef[(int64_t)rc * kCoefStride + 5 + 2 * tid];
-        ls.coef2[tid] = make_float4(re, re, im, im);
-    }
-    if (tid < kHid)  // e_c / 2 (exact)
-        reinterpret_cast<float *>(&ls.ec2[tid >> 1])[tid & 1] = L.ec ? 0.5f * L.ec[(int64_t)rc * kHid + tid] : 0.0f;
+    // item k of the launch: descriptor L.items[k], or k where every learned tile is shot
+    auto desc_of = [&](int64_t item) { return reinterpret_cast<const uint32_t *>(L.desc + (L.items ? L.items[item] : item)); };
+    constexpr int kDescWords = sizeof(TileDesc) / 4;
+    hist_zero<kLearnWin>(ls.hist);
+    if (tid < 3) ls.sred[tid] = 0u;
+    int64_t item = blockIdx.x;  // the queue hands out the items from gridDim.x on
+    if (tid < kDescWords && item < L.nitems) reinterpret_cast<uint32_t *>(&ls.desc[0])[tid] = desc_of(item)[tid];
     __syncthreads();
+    if (NET) umma::fence_after();
+    unsigned nb = 0, no = 0, nn = 0;
+    const float inv_cx = 1.0f / (float)(kTileX * L.cg.ktx), inv_cy = 1.0f / (float)(32 * L.cg.kty);
+    for (int cur = 0; item < L.nitems; cur ^= 1) {
+        const TileDesc &D = ls.desc[cur];
+        // warp 0 asks for the next item (read after the near field)
+        unsigned long long ticket = 0;
+        if (tid == 0) ticket = atomicAdd(L.counter, 1ull);
+        for (int q = tid; q < (int)(sizeof(CellRec) / 16); q += kThreads)
+            cp_async16(reinterpret_cast<float4 *>(&ls.cell) + q, reinterpret_cast<const float4 *>(L.cells + D.rc) + q);
 
-    // ray offsets from the tile centre: the high parts here, the low parts (LO) formed
-    // inside the near-field loop
-    float2 rx, ry[NP], px[NP], py[NP], Sx[NP], Sy[NP], Cx[NP], Cy[NP];
-    const float cxf = ts.tc[0], cyf = ts.tc[1];
-    if (LO) {
-        float h, l, h1, l1;
-        ray_offset((float)tx, ts.tc[2], ts.tc[8], R.dxh, R.dxl, h, l);
-        rx = f2(h, h);
+        // ray offsets from the tile centre: the high parts here, the low parts (LO) formed
+        // inside the near-field loop
+        float2 rx, ry[NP], px[NP], py[NP], Sx[NP], Sy[NP], Cx[NP], Cy[NP];
+        if (LO) {
+            float h, l, h1, l1;
+            ray_offset((float)tx, D.tc[2], D.tc[8], R.dxh, R.dxl, h, l);
+            rx = f2(h, h);
 #pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            float k0 = (float)(tg * 2 * NP + 2 * p), k1 = k0 + 1.0f;
-            ray_offset(k0, ts.tc[3], ts.tc[9], R.dyh, R.dyl, h, l);
-            ray_offset(k1, ts.tc[3], ts.tc[9], R.dyh, R.dyl, h1, l1);
-            ry[p] = f2(h, h1);
-            px[p] = py[p] = Sx[p] = Sy[p] = Cx[p] = Cy[p] = f2(0.f, 0.f);
-        }
-    } else {  // exact float offsets: e + k d with every step exact
-        const float kx = (float)tx;
-        const float dxr = __fmaf_rn(kx, R.dxh, ts.tc[2]);
-        rx = f2(dxr, dxr);
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            float k0 = (float)(tg * 2 * NP + 2 * p), k1 = k0 + 1.0f;
-            ry[p] = f2(__fmaf_rn(k0, R.dyh, ts.tc[3]), __fmaf_rn(k1, R.dyh, ts.tc[3]));
-            px[p] = py[p] = Sx[p] = Sy[p] = Cx[p] = Cy[p] = f2(0.f, 0.f);
-        }
-    }
-    // ---- near field: the 3 x 3 block's stars (about 1.3 per tile at the learned
-    // workload's density), staged 256 at a time and summed in compensated chunks
-    // of kNearChunk<NET> stars, padded with massless far stars
-    const int nnear = ls.nnear;
-    for (int base = 0; base < nnear; base += 256) {
-        constexpr int C = kNearChunk<NET>;
-        const int cnt = min(256, nnear - base), cntp = (cnt + C - 1) / C * C;
-        __syncthreads();
-        if (tid < cntp) {
-            float4 q = make_float4(kPadCoord, kPadCoord, 0.0f, 0.0f);
-            if (tid < cnt) {
-                int k = base + tid;
-                const int n0 = ls.re[0] - ls.rb[0], n1 = ls.re[1] - ls.rb[1];
-                const int idx = k < n0 ? ls.rb[0] + k : (k < n0 + n1 ? ls.rb[1] + (k - n0) : ls.rb[2] + (k - n0 - n1));
-                q = L.cstars[idx];
+            for (int p = 0; p < NP; ++p) {
+                float k0 = (float)(tg * 2 * NP + 2 * p), k1 = k0 + 1.0f;
+                ray_offset(k0, D.tc[3], D.tc[9], R.dyh, R.dyl, h, l);
+                ray_offset(k1, D.tc[3], D.tc[9], R.dyh, R.dyl, h1, l1);
+                ry[p] = f2(h, h1);
             }
-            const float nx = __fsub_rn(cxf, q.x), ny = __fsub_rn(cyf, q.y);
-            sm.st.q[0][tid] = make_float4(nx, nx, ny, ny);
-            sm.st.mm[0][tid] = f2(q.z, q.z);
+        } else {  // exact float offsets: e + k d with every step exact
+            const float dxr = __fmaf_rn((float)tx, R.dxh, D.tc[2]);
+            rx = f2(dxr, dxr);
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+                float k0 = (float)(tg * 2 * NP + 2 * p), k1 = k0 + 1.0f;
+                ry[p] = f2(__fmaf_rn(k0, R.dyh, D.tc[3]), __fmaf_rn(k1, R.dyh, D.tc[3]));
+            }
         }
-        __syncthreads();
-        const float4 *Q = sm.st.q[0];
-        const float2 *M = sm.st.mm[0];
-        {
+#pragma unroll
+        for (int p = 0; p < NP; ++p) Sx[p] = Sy[p] = Cx[p] = Cy[p] = f2(0.f, 0.f);
+        // ---- near field: the 3 x 3 block's stars, staged 256 at a time and summed in
+        // compensated chunks of kNearChunk<NET> stars
+        const int n0 = D.near_n[0], n1 = D.near_n[1], nnear = n0 + n1 + D.near_n[2];
+        for (int base = 0; base < nnear; base += 256) {
+            constexpr int C = kNearChunk<NET>;
+            const int cnt = min(256, nnear - base);
+            if (base) __syncthreads();  // the previous stage's reads are done
+            if (tid < cnt) {
+                const int k = base + tid;
+                const int at = k < n0 ? D.near_at[0] + k : (k < n0 + n1 ? D.near_at[1] + (k - n0) : D.near_at[2] + (k - n0 - n1));
+                const float4 q = L.cstars[at];
+                const float nx = __fsub_rn(D.tc[0], q.x), ny = __fsub_rn(D.tc[1], q.y);
+                near_st.q[0][tid] = make_float4(nx, nx, ny, ny);
+                near_st.mm[0][tid] = f2(q.z, q.z);
+            }
+            __syncthreads();
+            const float4 *Q = near_st.q[0];
+            const float2 *M = near_st.mm[0];
             float2 rxl = f2(0.f, 0.f), ryl[NP];
 #pragma unroll
             for (int p = 0; p < NP; ++p) ryl[p] = f2(0.f, 0.f);
             if (LO) {
                 float h, l, h1, l1;
-                ray_offset((float)tx, ts.tc[2], ts.tc[8], R.dxh, R.dxl, h, l);
+                ray_offset((float)tx, D.tc[2], D.tc[8], R.dxh, R.dxl, h, l);
                 rxl = f2(l, l);
 #pragma unroll
                 for (int p = 0; p < NP; ++p) {
                     float k0 = (float)(tg * 2 * NP + 2 * p), k1 = k0 + 1.0f;
-                    ray_offset(k0, ts.tc[3], ts.tc[9], R.dyh, R.dyl, h, l);
-                    ray_offset(k1, ts.tc[3], ts.tc[9], R.dyh, R.dyl, h1, l1);
+                    ray_offset(k0, D.tc[3], D.tc[9], R.dyh, R.dyl, h, l);
+                    ray_offset(k1, D.tc[3], D.tc[9], R.dyh, R.dyl, h1, l1);
                     ryl[p] = f2(l, l1);
                 }
             }
-            for (int k0 = 0; k0 < cntp; k0 += C) {
+#pragma unroll 1
+            for (int k0 = 0; k0 < cnt; k0 += C) {
+                const int k1 = min(k0 + C, cnt);
 #pragma unroll
-                for (int k = k0; k < k0 + C; ++k) {
+                for (int p = 0; p < NP; ++p) px[p] = py[p] = f2(0.f, 0.f);
+#pragma unroll 1
+                for (int k = k0; k < k1; ++k) {
                     const float4 q = Q[k];
                     const float2 m2 = M[k];
                     const float2 dx = LO ? __fadd2_rn(__fadd2_rn(rx, f2(q.x, q.y)), rxl) : __fadd2_rn(rx, f2(q.x, q.y));
@@ -1405,258 +1486,230 @@ __device__ __forceinline__ void learned_tile(const LearnedArgs &L, int bx, int b
                 for (int p = 0; p < NP; ++p) {
                     kahan2(Sx[p], Cx[p], px[p]);
                     kahan2(Sy[p], Cy[p], py[p]);
-                    px[p] = py[p] = f2(0.f, 0.f);
                 }
             }
         }
-    }
-    __syncthreads();  // star stages dead; the region now holds the network outputs
+        // the next item's descriptor, in flight until the binning
+        int64_t next = 0;
+        uint32_t dword = 0;
+        if (tid < 32) {
+            next = (int64_t)gridDim.x + (int64_t)__shfl_sync(0xffffffffu, ticket, 0);
+            if (tid < kDescWords && next < L.nitems) dword = desc_of(next)[tid];
+        }
+        asm volatile("cp.async.wait_all;\n" ::: "memory");
+        __syncthreads();  // the cell's record is in place; the near stage is dead (NET: the A operands' bytes)
 
-    // ---- network residual for the tile's 2048 rays (warp w: rays 256w .. 256w+255)
-    // the network's outputs (+ b3) for this thread's own rays, ray k at yv[2 k], yv[2 k + 1]
-    float yv[4 * NP];
-    const int ioff = (bx % cg.ktx) * kTileX, joff = (by % cg.kty) * kTileY;
-    const float inv_cx = 1.0f / (float)(kTileX * cg.ktx), inv_cy = 1.0f / (float)(kTileY * cg.kty);
-    if (NET) {
-        // Two warpgroups; warpgroup wg takes the 128-ray chunks wg, wg + 2, ...  Each
-        // thread writes its ray's layer-1 activations (BF16) as row t of the
-        // warpgroup's A operand; one thread issues h2 = A W2^T on the tensor cores
-        // (tcgen05.mma, M = 128, N = 64, K = 64 in four K = 16 steps, FP32
-        // accumulator in tensor memory) and commits to the warpgroup's mbarrier;
-        // then each thread reads its ray's 64 accumulators back and finishes SiLU
-        // and layer 3 in registers.
-        const int warp = tid >> 5, lane = tid & 31, wg = warp >> 2, t = tid & 127;
-        unsigned char *abuf = abuf_all + wg * kTcABytes;
-        const uint32_t dcol = ls.tmem + (uint32_t)(wg * kHid);
-        const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        constexpr uint32_t idesc = umma::idesc_bf16(kTcChunk, kHid);
+        // ---- network residual for the tile's 2048 rays
+        // the network's outputs (+ b3) for this thread's own rays, ray k at yv[2 k], yv[2 k + 1]
+        float yv[4 * NP];
+        const int ioff = D.ioff, joff = D.joff;
+        if (NET) {
+            // Two warpgroups; warpgroup wg takes the 128-ray chunks wg, wg + 2, ...  Each
+            // thread writes its ray's layer-1 activations (BF16) as row t of the
+            // warpgroup's A operand; one thread issues h2 = A W2^T on the tensor cores
+            // (tcgen05.mma, M = 128, N = 64, K = 64 in four K = 16 steps, FP32
+            // accumulator in tensor memory) and commits to the warpgroup's mbarrier;
+            // then each thread reads its ray's 64 accumulators back and finishes SiLU
+            // and layer 3 in registers.
+            const int warp = tid >> 5, lane = tid & 31, wg = warp >> 2, t = tid & 127;
+            unsigned char *abuf = dyn_smem + wg * kTcABytes;
+            const uint32_t dcol = ls.tmem + (uint32_t)(wg * kHid);
+            const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
+            constexpr uint32_t idesc = umma::idesc_bf16(kTcChunk, kHid);
 #pragma unroll 1
-        for (int k = 0; k < 2 * NP; ++k) {  // chunk k: ray k of each thread of the warpgroup
-            const int row = tg * 2 * NP + k;  // the ray's row in the tile (its column is tx)
-            float y0 = 0.0f, y1 = 0.0f;
-            if (!ls.tc_dead[wg]) {
-                const float ux = (float)(2 * (ioff + tx) + 1) * inv_cx - 1.0f;
-                const float uy = (float)(2 * (joff + row) + 1) * inv_cy - 1.0f;
-                const float2 uxx = make_float2(ux, ux), uyy = make_float2(uy, uy);
+            for (int k = 0; k < 2 * NP; ++k) {  // chunk k: ray k of each thread of the warpgroup
+                const int row = tg * 2 * NP + k;  // the ray's row in the tile (its column is tx)
+                float y0 = 0.0f, y1 = 0.0f;
+                if (!ls.tc_dead[wg]) {
+                    const float ux = (float)(2 * (ioff + tx) + 1) * inv_cx - 1.0f;
+                    const float uy = (float)(2 * (joff + row) + 1) * inv_cy - 1.0f;
+                    const float2 uxx = make_float2(ux, ux), uyy = make_float2(uy, uy);
 #pragma unroll
-                for (int k8 = 0; k8 < kHid / 8; ++k8) {
-                    uint32_t pk[4];
+                    for (int k8 = 0; k8 < kHid / 8; ++k8) {
+                        uint32_t pk[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {  // units 8 k8 + 2 q and + 1
-                        const float2 e = ls.ec2[4 * k8 + q];
-                        const float4 w = L.net.w1u[4 * k8 + q];
-                        // (e_c + W1u[.][0] ux + W1u[.][1] uy) / 2, then SiLU, for both units
-                        float2 v = __ffma2_rn(make_float2(w.x, w.y), uxx, e);
-                        v = __ffma2_rn(make_float2(w.z, w.w), uyy, v);
-                        const float2 a = silu_half2(v);
-                        pk[q] = pack_bf16(a.x, a.y);
-                    }
-                    *reinterpret_cast<uint4 *>(abuf + umma::cm_offset(t, k8 * 8)) =
-                        make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                }
-                umma::fence_async_smem();
-                umma::fence_before();
-                umma::wg_sync(wg);
-                umma::fence_after();
-                if (t == 0) {
-#pragma unroll
-                    for (int ks = 0; ks < kHid / 16; ++ks)
-                        umma::mma_bf16(dcol, umma::desc(umma::smem_addr(abuf) + ks * 256, 128, 1024),
-                                       umma::desc(umma::smem_addr(ls.w2cm) + ks * 256, 128, 1024), idesc,
-                                       ks > 0 ? 1u : 0u);
-                    umma::commit(&ls.mbar[wg]);
-                }
-                // (the wait probe, a test aid, polls ls.idle instead: the wait runs out and
-                // the warpgroup takes the failure path below)
-                const bool ok = __all_sync(0xffffffffu, L.wait_probe ? umma::mbar_wait(&ls.idle, 0, kProbePolls)
-                                                                     : umma::mbar_wait(&ls.mbar[wg], phase, kWaitPolls));
-                if (lane == 0) ls.wg_ok[warp] = ok ? 1 : 0;
-                umma::wg_sync(wg);
-                const bool wg_ok = ls.wg_ok[4 * wg] && ls.wg_ok[4 * wg + 1] && ls.wg_ok[4 * wg + 2] &&
-                                   ls.wg_ok[4 * wg + 3];
-                if (wg_ok) {
-                    phase ^= 1u;
-                    umma::fence_after();
-                    // layer 2's bias and SiLU, and layer 3, two units at a time (even and
-                    // odd units summed apart, then added)
-                    float2 y0p = make_float2(0.0f, 0.0f), y1p = make_float2(0.0f, 0.0f);
-#pragma unroll
-                    for (int c0 = 0; c0 < kHid; c0 += 16) {
-                        uint32_t acc[16];
-                        umma::ld16(dcol + lane_base + (uint32_t)c0, acc);
-#pragma unroll
-                        for (int j = 0; j < 16; j += 2) {
-                            const float4 qa = L.net.l2p[(c0 + j) >> 1];
-                            const float2 qb = L.net.l2q[(c0 + j) >> 1];
-                            const float2 a2 = silu_half2(__fadd2_rn(
-                                make_float2(__uint_as_float(acc[j]), __uint_as_float(acc[j + 1])), make_float2(qa.x, qa.y)));
-                            y0p = __ffma2_rn(make_float2(qa.z, qa.w), a2, y0p);
-                            y1p = __ffma2_rn(qb, a2, y1p);
+                        for (int q = 0; q < 4; ++q) {  // units 8 k8 + 2 q and + 1
+                            const float2 e = ls.cell.ec[4 * k8 + q];
+                            const float4 w = L.net.w1u[4 * k8 + q];
+                            // (e_c + W1u[.][0] ux + W1u[.][1] uy) / 2, then SiLU, for both units
+                            float2 v = __ffma2_rn(make_float2(w.x, w.y), uxx, e);
+                            v = __ffma2_rn(make_float2(w.z, w.w), uyy, v);
+                            const float2 a = silu_half2(v);
+                            pk[q] = pack_bf16(a.x, a.y);
                         }
+                        *reinterpret_cast<uint4 *>(abuf + umma::cm_offset(t, k8 * 8)) =
+                            make_uint4(pk[0], pk[1], pk[2], pk[3]);
                     }
-                    y0 = y0p.x + y0p.y;
-                    y1 = y1p.x + y1p.y;
-                } else if (t == 0) {
-                    // the MMAs never reported completion: stop using the tensor path,
-                    // remember the phase to drain before tensor memory is freed
-                    ls.tc_dead[wg] = 1;
-                    ls.pending[wg] = phase;
-                    atomicExch(L.err, 1);
+                    umma::fence_async_smem();
+                    umma::fence_before();
+                    umma::wg_sync(wg);
+                    umma::fence_after();
+                    if (t == 0) {
+#pragma unroll
+                        for (int ks = 0; ks < kHid / 16; ++ks)
+                            umma::mma_bf16(dcol, umma::desc(umma::smem_addr(abuf) + ks * 256, 128, 1024),
+                                           umma::desc(umma::smem_addr(ls.w2cm) + ks * 256, 128, 1024), idesc,
+                                           ks > 0 ? 1u : 0u);
+                        umma::commit(&ls.mbar[wg]);
+                    }
+                    // (the wait probe, a test aid, polls ls.idle instead: the wait runs out and
+                    // the warpgroup takes the failure path below)
+                    const bool ok = __all_sync(0xffffffffu, L.wait_probe ? umma::mbar_wait(&ls.idle, 0, kProbePolls)
+                                                                         : umma::mbar_wait(&ls.mbar[wg], phase, kWaitPolls));
+                    if (lane == 0) ls.wg_ok[warp] = ok ? 1 : 0;
+                    umma::wg_sync(wg);
+                    const bool wg_ok = ls.wg_ok[4 * wg] && ls.wg_ok[4 * wg + 1] && ls.wg_ok[4 * wg + 2] &&
+                                       ls.wg_ok[4 * wg + 3];
+                    if (wg_ok) {
+                        phase ^= 1u;
+                        umma::fence_after();
+                        // layer 2's bias and SiLU, and layer 3, two units at a time (even and
+                        // odd units summed apart, then added)
+                        float2 y0p = make_float2(0.0f, 0.0f), y1p = make_float2(0.0f, 0.0f);
+#pragma unroll
+                        for (int c0 = 0; c0 < kHid; c0 += 16) {
+                            uint32_t acc[16];
+                            umma::ld16(dcol + lane_base + (uint32_t)c0, acc);
+#pragma unroll
+                            for (int j = 0; j < 16; j += 2) {
+                                const float4 qa = L.net.l2p[(c0 + j) >> 1];
+                                const float2 qb = L.net.l2q[(c0 + j) >> 1];
+                                const float2 a2 = silu_half2(__fadd2_rn(
+                                    make_float2(__uint_as_float(acc[j]), __uint_as_float(acc[j + 1])), make_float2(qa.x, qa.y)));
+                                y0p = __ffma2_rn(make_float2(qa.z, qa.w), a2, y0p);
+                                y1p = __ffma2_rn(qb, a2, y1p);
+                            }
+                        }
+                        y0 = y0p.x + y0p.y;
+                        y1 = y1p.x + y1p.y;
+                    } else if (t == 0) {
+                        // the MMAs never reported completion: stop using the tensor path,
+                        // remember the phase to drain before tensor memory is freed
+                        ls.tc_dead[wg] = 1;
+                        ls.pending[wg] = phase;
+                        atomicExch(L.err, 1);
+                    }
+                    umma::fence_before();
+                    umma::wg_sync(wg);  // accumulators read and A consumed before the next chunk
                 }
-                umma::fence_before();
-                umma::wg_sync(wg);  // accumulators read and A consumed before the next chunk
+                yv[2 * k] = y0 + L.net.b3[0];
+                yv[2 * k + 1] = y1 + L.net.b3[1];
             }
-            yv[2 * k] = y0 + L.net.b3[0];
-            yv[2 * k + 1] = y1 + L.net.b3[1];
         }
-    }
-
-    // ---- far field and beta per ray, the two rays of each pair (rows 2p and 2p + 1 of
-    // column tx) in the two lanes of f32x2 registers: the same operations per ray as a
-    // scalar loop, x - y as fma(y, -1, x) (one rounding, as a subtraction)
-    float bxh[2 * NP], byh[2 * NP], bxl[2 * NP], byl[2 * NP];
-    {
-        const float2 m1 = make_float2(-1.0f, -1.0f);
-        auto sub2 = [&](float2 x, float2 y) { return __ffma2_rn(y, m1, x); };
-        auto two_sum2 = [&](float2 a, float2 b, float2 &s, float2 &e) {  // Knuth's TwoSum per lane
-            const float2 x = __fadd2_rn(a, b), bb = sub2(x, a);
-            e = __fadd2_rn(sub2(a, sub2(x, bb)), sub2(b, bb));
-            s = x;
-        };
-        auto dup = [](float x) { return make_float2(x, x); };
-        const float uxr = (float)(2 * (ioff + tx) + 1) * inv_cx - 1.0f;
-        const float2 vx = dup(uxr * 0.70710678f);
-        const float2 tc4 = dup(ts.tc[4]), tc5 = dup(ts.tc[5]), tc6 = dup(ts.tc[6]), tc7 = dup(ts.tc[7]);
-        const float2 nb0x = dup(-ls.coef[0]), b0y = dup(ls.coef[1]), b1x = dup(ls.coef[2]), b1y = dup(ls.coef[3]);
-        const float2 fa11 = dup(a.lens.fa11), fa12 = dup(a.lens.fa12), fa22 = dup(a.lens.fa22);
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-            const int jl = tg * 2 * NP + 2 * p;  // the pair's first row in the tile
-            const float uy0 = (float)(2 * (joff + jl) + 1) * inv_cy - 1.0f;
-            const float uy1 = (float)(2 * (joff + jl + 1) + 1) * inv_cy - 1.0f;
-            const float2 vy = make_float2(uy0 * 0.70710678f, uy1 * 0.70710678f);
-            const float2 nvy = make_float2(-vy.x, -vy.y);
-            // T = sum_{q=1}^{pe} b_q v^q + v^(pe+1) q_net, q_net = s_c (network output) or 0:
-            // Horner with q_net as the innermost coefficient; (ar, ai) = T's real and
-            // imaginary parts for the two rays
-            float2 ar = make_float2(0.f, 0.f), ai = make_float2(0.f, 0.f);
-            if (L.use_net) {
-                ar = make_float2(ls.sc * yv[4 * p], ls.sc * yv[4 * p + 2]);
-                ai = make_float2(ls.sc * yv[4 * p + 1], ls.sc * yv[4 * p + 3]);
-            }
-            auto cmul2 = [&]() {  // (ar + i ai) (vx + i vy)
-                const float2 t = __fmul2_rn(ar, vx), u = __fmul2_rn(ar, vy);
-                ar = __ffma2_rn(ai, nvy, t);
-                ai = __ffma2_rn(ai, vx, u);
+        // ---- far field and beta per ray, the two rays of each pair (rows 2p and 2p + 1 of
+        // column tx) in the two lanes of f32x2 registers: the same operations per ray as a
+        // scalar loop, x - y as fma(y, -1, x) (one rounding, as a subtraction)
+        float bxh[2 * NP], byh[2 * NP], bxl[2 * NP], byl[2 * NP];
+        {
+            const float2 m1 = make_float2(-1.0f, -1.0f);
+            auto sub2 = [&](float2 x, float2 y) { return __ffma2_rn(y, m1, x); };
+            auto two_sum2 = [&](float2 a, float2 b, float2 &s, float2 &e) {  // Knuth's TwoSum per lane
+                const float2 x = __fadd2_rn(a, b), bb = sub2(x, a);
+                e = __fadd2_rn(sub2(a, sub2(x, bb)), sub2(b, bb));
+                s = x;
             };
-            cmul2();
-            for (int q = L.pe; q >= 1; --q) {
-                const float4 c = ls.coef2[q - 1];
-                ar = __fadd2_rn(ar, make_float2(c.x, c.y));
-                ai = __fadd2_rn(ai, make_float2(c.z, c.w));
-                cmul2();
-            }
-            // A delta from the offsets' high parts: the low parts (2^-24 of an offset)
-            // matter only inside the near-field sum, next to a star
-            const float2 lx = __ffma2_rn(fa11, rx, __fmul2_rn(fa12, ry[p]));
-            const float2 ly = __ffma2_rn(fa12, rx, __fmul2_rn(fa22, ry[p]));
-            // alpha_far = (Re F, -Im F) + residual;  F = b0 + T
-            float2 th, tl, t2, small, h, l;
-            two_sum2(tc4, __fmul2_rn(Sx[p], m1), th, tl);
-            two_sum2(th, nb0x, th, t2);
-            small = __fadd2_rn(__fadd2_rn(tc6, Cx[p]), lx);
-            small = sub2(small, __fadd2_rn(b1x, ar));
-            tl = __fadd2_rn(__fadd2_rn(tl, t2), small);
-            two_sum2(th, tl, h, l);
-            bxh[2 * p] = h.x, bxh[2 * p + 1] = h.y, bxl[2 * p] = l.x, bxl[2 * p + 1] = l.y;
-            two_sum2(tc5, __fmul2_rn(Sy[p], m1), th, tl);
-            two_sum2(th, b0y, th, t2);
-            small = __fadd2_rn(__fadd2_rn(tc7, Cy[p]), ly);
-            small = __fadd2_rn(small, __fadd2_rn(b1y, ai));
-            tl = __fadd2_rn(__fadd2_rn(tl, t2), small);
-            two_sum2(th, tl, h, l);
-            byh[2 * p] = h.x, byh[2 * p + 1] = h.y, byl[2 * p] = l.x, byl[2 * p + 1] = l.y;
-        }
-    }
-
-    // ---- binning (the epilogue of the plain kernel)
-    const int ix = i0 + tx;
-    const bool col_ok = ix < R.nx;
-    __syncthreads();
-    hist_zero(sm.hist);
-    if (tid == kThreads / 2 + kTileX / 2) {  // the tile's middle ray
-        ts.win[0] = win_origin(pair_axis_rough(bxh[0], a.bin.ax), a.bin.nx);
-        ts.win[1] = win_origin(pair_axis_rough(byh[0], a.bin.ay), a.bin.ny);
-    }
-    __syncthreads();
-    const WinHist<> W = make_window(sm.hist, ts.win[0], ts.win[1], a.bin);
-    const int nrow = col_ok ? min(2 * NP, R.ny - (j0 + tg * 2 * NP)) : 0;  // this thread's rays in the grid
-    unsigned no = 0, nn = 0;
+            auto dup = [](float x) { return make_float2(x, x); };
+            const float uxr = (float)(2 * (ioff + tx) + 1) * inv_cx - 1.0f;
+            const float2 vx = dup(uxr * 0.70710678f);
+            constexpr int G = 2;             // pairs evaluated together: they share the coefficients' loads
+            constexpr int kQ = NET ? 1 : 4;  // orders unrolled
 #pragma unroll
-    for (int r = 0; r < 2 * NP; ++r) {
-        if (r < nrow) {
-            bin_pair<true>(bxh[r], byh[r], bxl[r], byl[r], a.bin, W, a.counts, no, nn);
-            if (a.beta_out) {
-                float4 *bo = reinterpret_cast<float4 *>(a.beta_out);
-                bo[(int64_t)(j0 + tg * 2 * NP + r) * R.nx + ix] = make_float4(bxh[r], byh[r], bxl[r], byl[r]);
+            for (int p0 = 0; p0 < NP; p0 += G) {
+                // T = sum_{q=1}^{pe} b_q v^q + v^(pe+1) q_net, q_net = s_c (network output) or 0:
+                // Horner with q_net as the innermost coefficient; (ar, ai) = T's real and
+                // imaginary parts for the two rays
+                float2 vy[G], nvy[G], ar[G], ai[G];
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const int p = p0 + g, jl = tg * 2 * NP + 2 * p;  // the pair's first row in the tile
+                    const float uy0 = (float)(2 * (joff + jl) + 1) * inv_cy - 1.0f;
+                    const float uy1 = (float)(2 * (joff + jl + 1) + 1) * inv_cy - 1.0f;
+                    vy[g] = make_float2(uy0 * 0.70710678f, uy1 * 0.70710678f);
+                    nvy[g] = make_float2(-vy[g].x, -vy[g].y);
+                    ar[g] = ai[g] = make_float2(0.f, 0.f);
+                    if (NET) {
+                        const float sc = ls.cell.sc.x;
+                        ar[g] = make_float2(sc * yv[4 * p], sc * yv[4 * p + 2]);
+                        ai[g] = make_float2(sc * yv[4 * p + 1], sc * yv[4 * p + 3]);
+                    }
+                }
+                auto cmul2 = [&]() {  // (ar + i ai) (vx + i vy)
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        const float2 t = __fmul2_rn(ar[g], vx), u = __fmul2_rn(ar[g], vy[g]);
+                        ar[g] = __ffma2_rn(ai[g], nvy[g], t);
+                        ai[g] = __ffma2_rn(ai[g], vx, u);
+                    }
+                };
+                if (NET) cmul2();  // (zero times v without the network)
+#pragma unroll kQ
+                for (int q = L.pe; q >= 1; --q) {
+                    const float4 c = ls.cell.b[q - 1];
+#pragma unroll
+                    for (int g = 0; g < G; ++g) {
+                        ar[g] = __fadd2_rn(ar[g], make_float2(c.x, c.y));
+                        ai[g] = __fadd2_rn(ai[g], make_float2(c.z, c.w));
+                    }
+                    cmul2();
+                }
+                const float4 b0 = ls.cell.b0;
+                const float2 fa11 = dup(a.lens.fa11), fa12 = dup(a.lens.fa12), fa22 = dup(a.lens.fa22);
+#pragma unroll
+                for (int g = 0; g < G; ++g) {
+                    const int p = p0 + g;
+                    // A delta from the offsets' high parts: the low parts (2^-24 of an offset)
+                    // matter only inside the near-field sum, next to a star
+                    const float2 lx = __ffma2_rn(fa11, rx, __fmul2_rn(fa12, ry[p]));
+                    const float2 ly = __ffma2_rn(fa12, rx, __fmul2_rn(fa22, ry[p]));
+                    // alpha_far = (Re F, -Im F) + residual;  F = b0 + T
+                    float2 th, tl, t2, small, h, l;
+                    two_sum2(dup(D.tc[4]), __fmul2_rn(Sx[p], m1), th, tl);
+                    two_sum2(th, dup(-b0.x), th, t2);
+                    small = __fadd2_rn(__fadd2_rn(dup(D.tc[6]), Cx[p]), lx);
+                    small = sub2(small, __fadd2_rn(dup(b0.z), ar[g]));
+                    tl = __fadd2_rn(__fadd2_rn(tl, t2), small);
+                    two_sum2(th, tl, h, l);
+                    bxh[2 * p] = h.x, bxh[2 * p + 1] = h.y, bxl[2 * p] = l.x, bxl[2 * p + 1] = l.y;
+                    two_sum2(dup(D.tc[5]), __fmul2_rn(Sy[p], m1), th, tl);
+                    two_sum2(th, dup(b0.y), th, t2);
+                    small = __fadd2_rn(__fadd2_rn(dup(D.tc[7]), Cy[p]), ly);
+                    small = __fadd2_rn(small, __fadd2_rn(dup(b0.w), ai[g]));
+                    tl = __fadd2_rn(__fadd2_rn(tl, t2), small);
+                    two_sum2(th, tl, h, l);
+                    byh[2 * p] = h.x, byh[2 * p + 1] = h.y, byl[2 * p] = l.x, byl[2 * p + 1] = l.y;
+                }
             }
         }
-    }
-    const unsigned nb = (unsigned)max(nrow, 0) - no - nn;
-    __syncthreads();
-    hist_flush(W, a.bin, a.counts);
-    stats_add_block(nb, no, nn, ts.sred, a.stats);
-}
 
-// NET: the network on the tensor cores (tcgen05; 128 tensor-memory columns and the
-// two A operands in dynamic shared memory, in the same bytes as the star stage and
-// window); without it (the series alone) the kernel carries no tensor-core code.
-template <bool NET, bool LO>
-// Four CTAs per SM (64 registers, ~280 bytes of spills per thread; tensor memory
-// holds four CTAs' 128 columns): eight warps per scheduler hide the latency of the
-// 128 hardware tanh per ray.  Measured per 32768^2-ray map: two CTAs per SM 0.060 s,
-// three 0.056 s (when first measured); three 44.8 ms, four 44.0 ms with the current
-// network block, and 13.2 -> 11.8 ms for the order-16 series alone.
-__global__ void __launch_bounds__(kThreads, 4) k_shoot_learned(LearnedArgs L)
-{
-    __shared__ TileShared ts;
-    __shared__ __align__(128) LearnSmem ls;
-    __shared__ long long s_item;
-    // dynamic: the star stage and window of the tile phases without tensor-core work,
-    // and (NET) the two A operands of the network phase in the same bytes
-    extern __shared__ __align__(128) unsigned char dyn_smem[];
-    LearnTileSmem &sm = *reinterpret_cast<LearnTileSmem *>(dyn_smem);
-    unsigned char *tc_abuf = dyn_smem;
-    const int tid = threadIdx.x;
-    uint32_t phase = 0;  // completed MMA batches of this thread's warpgroup, mod 2
-    if (NET) {
-        for (int i = tid; i < kHid * kHid; i += kThreads)
-            *reinterpret_cast<__nv_bfloat16 *>(ls.w2cm + umma::cm_offset(i / kHid, i % kHid)) =
-                __float2bfloat16_rn(0.5f * __bfloat162float(L.w2b[i]));  // W2 / 2 (exact)
-        if (tid < 2) ls.tc_dead[tid] = 0;
-        if (tid == 0) {
-            umma::mbar_init(&ls.mbar[0], 1);
-            umma::mbar_init(&ls.mbar[1], 1);
-            umma::mbar_init(&ls.idle, 1);
-            umma::fence_mbar_init();
+        // ---- binning
+        const int ix = D.bx * kTileX + tx, jy = D.by * 32 + tg * 2 * NP;
+        const int nrow = ix < R.nx ? min(2 * NP, R.ny - jy) : 0;  // this thread's rays in the grid
+        if (tid < 32) {
+            if (tid < kDescWords) reinterpret_cast<uint32_t *>(&ls.desc[cur ^ 1])[tid] = dword;
+            if (tid == 0) ls.first = next;
         }
-        if (tid < 32) umma::tmem_alloc(&ls.tmem, 2 * kHid);
-        umma::fence_async_smem();  // W2 is read by the tensor cores
-        umma::fence_before();
+        if (tid == kThreads / 2 + kTileX / 2) {  // the tile's middle ray
+            ls.win[0] = win_origin<kLearnWin>(pair_axis_rough(bxh[0], a.bin.ax), a.bin.nx);
+            ls.win[1] = win_origin<kLearnWin>(pair_axis_rough(byh[0], a.bin.ay), a.bin.ny);
+        }
         __syncthreads();
-        umma::fence_after();
+        item = ls.first;
+        const WinHist<kLearnWin> W = make_window<kLearnWin>(ls.hist, ls.win[0], ls.win[1], a.bin);
+#pragma unroll
+        for (int r = 0; r < 2 * NP; ++r) {
+            if (r < nrow) {
+                bin_pair<true>(bxh[r], byh[r], bxl[r], byl[r], a.bin, W, a.counts, no, nn);
+                if (a.beta_out) {
+                    float4 *bo = reinterpret_cast<float4 *>(a.beta_out);
+                    bo[(int64_t)(jy + r) * R.nx + ix] = make_float4(bxh[r], byh[r], bxl[r], byl[r]);
+                }
+            }
+        }
+        nb += (unsigned)max(nrow, 0);
+        __syncthreads();
+        hist_flush<true>(W, a.bin, a.counts);
     }
-    const int ntx = (L.plain.rays.nx + kTileX - 1) / kTileX;
-    for (;;) {
-        __syncthreads();
-        if (tid == 0) s_item = (long long)atomicAdd(L.counter, 1ull);
-        __syncthreads();
-        const int64_t item = s_item;
-        if (item >= L.nitems) break;
-        const int tile = L.items[item];
-        const int bx = tile % ntx, by = tile / ntx;
-        learned_tile<NET, LO>(L, bx, by, sm, ts, ls, tc_abuf, phase);
-    }
+    stats_add_block(nb - no - nn, no, nn, ls.sred, a.stats);
     if (NET) {
         // a warpgroup that gave up on a wait drains its MMAs (again bounded) before
         // the tensor memory is freed
@@ -1693,7 +1746,7 @@ cudaError_t ff_learned_grid(int *grid)
     // beyond those resident only find the shared work queue empty.
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_shoot_learned<false, false>, kThreads,
-                                                                  sizeof(LearnTileSmem));
+                                                                  sizeof(NearStage));
     if (e != cudaSuccess) return e;
     int dev = 0, nsm = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1710,7 +1763,7 @@ static cudaError_t launch_learned_t(const LearnedArgs &L, unsigned g, cudaStream
         if (e != cudaSuccess) return e;
         k_shoot_learned<true, LO><<<g, kThreads, kLearnedDynSmem, s>>>(L);
     } else {
-        k_shoot_learned<false, LO><<<g, kThreads, sizeof(LearnTileSmem), s>>>(L);
+        k_shoot_learned<false, LO><<<g, kThreads, sizeof(NearStage), s>>>(L);
     }
     return cudaGetLastError();
 }

@@ -52,20 +52,33 @@ struct NetConsts {
     float b3[2];
 };
 
+// One learned tile (k_tile_desc) and one cell (k_cell_rec), as the kernel takes them.
+struct TileDesc {
+    float tc[10];      // centre, first ray's offset, A c high and low, the offset's low parts (x, y each)
+    int near_at[3], near_n[3];  // near stars: runs in cstars
+    int bx, by;        // tile column and row
+    int rc;            // ray cell
+    int ioff, joff;    // first ray's column and row within the cell
+    int pad;
+};
+struct CellRec {
+    float4 b0;         // {Re, Im} high, {Re, Im} low
+    float4 b[kPeMax];  // b_q as {Re, Re, Im, Im}: both rays of a pair at once
+    float4 sc;         // {s_c, -, -, -}
+    float2 ec[kNetPairs];  // {e_c, e_c+1} / 2: the embedding of hidden units c, c + 1
+};
+
 // Everything the learned shooting kernel reads.
 struct LearnedArgs {
     ShootArgs plain;           // grids, lens terms, counts, counters
     CellGrid cg;
-    const int *cstart;         // extended cells + 1: CSR offsets into cstars
     const float4 *cstars;      // stars sorted by extended cell (input order within a cell)
-    const float *coef;         // per ray cell kCoefStride floats
-    const float *sc;           // per ray cell residual bound s_c
-    const float *ec;           // per ray cell 64 floats: bf16(W1z) bf16(z_c) + b1
-    const float *params;       // FP32 network parameters (flat layout of mlp.cuh)
+    const TileDesc *desc;      // tiles of the cells that passed validation
+    const CellRec *cells;      // per ray cell
     const __nv_bfloat16 *w2b;  // W2 in BF16, [out][in]
     int pe;
     int use_net;
-    const int *items;          // tile index per work item (tiles of cells that passed validation)
+    const int *items;          // descriptor per work item (nullptr: item k is descriptor k)
     int64_t nitems;
     unsigned long long *counter;
     int *err;                  // set to 1 if a tensor-core completion wait gave up (results invalid)
@@ -154,6 +167,9 @@ cudaError_t ff_embed(const float *params, const float *z, int nrc, float *ec, cu
 cudaError_t ff_flags(const unsigned *maxerr, int nrc, float tol, int *flags, cudaStream_t s);
 cudaError_t ff_shoot_learned(const LearnedArgs &L, int grid, cudaStream_t s);
 cudaError_t ff_learned_grid(int *grid);
+cudaError_t ff_tile_desc(const int *tiles, int64_t n, const RayGrid &rays, const LensTerms &lens, const CellGrid &cg,
+                         const int *cstart, TileDesc *out, cudaStream_t s);
+cudaError_t ff_cell_rec(const float *coef, const float *sc, const float *ec, int nrc, CellRec *out, cudaStream_t s);
 // The learned kernel's NetConsts from the flat FP32 parameters (host copy).
 void ff_net_consts(const float *params_host, NetConsts *out);
 

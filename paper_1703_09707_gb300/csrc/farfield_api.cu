@@ -43,7 +43,9 @@ struct FarState {
     int *items = nullptr;
     int64_t nitems = 0, nfallback_tiles = 0;
     std::vector<int> h_items;      // host copy of the work list
-    int *sub_items = nullptr;      // filtered work list for row-restricted calls
+    int *sub_items = nullptr;      // row-restricted calls: fallback tiles, then learned tiles' descriptors
+    TileDesc *desc = nullptr;      // the learned tiles, in the work list's order
+    CellRec *cells = nullptr;      // the ray cells
     unsigned long long *counter = nullptr;
     int *d_err = nullptr;  // learned kernel: a tensor-core wait gave up
     int grid = 0;
@@ -86,7 +88,7 @@ void free_state(FarState *f)
     ffree(f->params), ffree(f->m), ffree(f->v), ffree(f->grads), ffree(f->loss);
     ffree(f->w1zb), ffree(f->w2b), ffree(f->wimg), ffree(f->ec), ffree(f->flags);
     ffree(f->vmax_net), ffree(f->vmax_series), ffree(f->vsum), ffree(f->items), ffree(f->counter);
-    ffree(f->sub_items);
+    ffree(f->sub_items), ffree(f->desc), ffree(f->cells);
     ffree(f->gpart), ffree(f->dzs), ffree(f->d_err);
     f->gpart_rows = f->dzs_samples = 0;
     f->ready = false;
@@ -150,6 +152,7 @@ int alloc_state(FarState *f, int64_t nstars)
     FCUDA(dmalloc(&f->w2b, sizeof(__nv_bfloat16) * mlp::kHid * mlp::kHid), "cudaMalloc");
     FCUDA(dmalloc(&f->wimg, (size_t)ff_weight_image_bytes()), "cudaMalloc");
     FCUDA(dmalloc(&f->ec, sizeof(float) * (size_t)nrc * mlp::kHid), "cudaMalloc");
+    FCUDA(dmalloc(&f->cells, sizeof(CellRec) * (size_t)nrc), "cudaMalloc");
     FCUDA(dmalloc(&f->flags, sizeof(int) * nrc), "cudaMalloc");
     FCUDA(dmalloc(&f->vmax_net, sizeof(unsigned) * nrc), "cudaMalloc");
     FCUDA(dmalloc(&f->vmax_series, sizeof(unsigned) * nrc), "cudaMalloc");
@@ -216,7 +219,7 @@ int validate(FarState *f, int64_t per_cell, uint64_t seed, cudaStream_t s, doubl
 
 // Flags from the per-cell validation maxima, then the work list: tiles of flagged
 // cells (exact direct sum, heavy) first, then the rest.
-int schedule(FarState *f, cudaStream_t s)
+int schedule(const mlens_ctx *ctx, FarState *f, cudaStream_t s)
 {
     const unsigned *src = f->use_net ? f->vmax_net : f->vmax_series;
     FCUDA(ff_flags(src, f->nrc, (float)f->tol, f->flags, s), "flags");
@@ -242,6 +245,11 @@ int schedule(FarState *f, cudaStream_t s)
     FCUDA(cudaMemcpy(f->items, heavy.data(), sizeof(int) * f->nitems, cudaMemcpyHostToDevice), "memcpy(items)");
     f->h_items = heavy;
     ffree(f->sub_items);
+    const int64_t nlearned = f->nitems - f->nfallback_tiles;
+    ffree(f->desc);
+    FCUDA(dmalloc(&f->desc, sizeof(TileDesc) * std::max<int64_t>(nlearned, 1)), "cudaMalloc(tile descriptors)");
+    FCUDA(ff_tile_desc(f->items + f->nfallback_tiles, nlearned, make_ray_grid(f->rays), ctx->lens, f->cg, f->start,
+                       f->desc, s), "tile descriptors");
     int nflag = 0;
     double mx_n = 0.0, mx_s = 0.0;
     for (int i = 0; i < f->nrc; ++i) {
@@ -273,6 +281,7 @@ int finish_inference_tables(FarState *f, cudaStream_t s)
 {
     FCUDA(ff_prep_bf16(f->params, f->w1zb, f->w2b, f->wimg, s), "prep");
     FCUDA(ff_embed(f->params, f->params + mlp::kParams, f->nrc, f->ec, s), "embed");
+    FCUDA(ff_cell_rec(f->coef, f->sc, f->ec, f->nrc, f->cells, s), "cell records");
     return MLENS_OK;
 }
 
@@ -437,7 +446,7 @@ int mlens_fit_far_field(mlens_ctx *ctx, const mlens_grid *rays, const mlens_fit_
     }
     f->report.val_mean_err_net = f->use_net ? mn : -1.0;
     f->report.val_mean_err_series = ms;
-    if ((rc = schedule(f, s))) return rc;
+    if ((rc = schedule(ctx, f, s))) return rc;
     if ((rc = finish_inference_tables(f, s))) return rc;
     FCUDA(cudaStreamSynchronize(s), "sync");
     f->report.seconds_validate = now_s() - t2;
@@ -478,8 +487,9 @@ int mlens_shoot_learned(mlens_ctx *ctx, const mlens_grid *rays, const mlens_grid
             const int t = f->h_items[q];
             const int by = t / ntx;
             if (by * 32 >= row_begin && by * 32 < row_end) {
-                sub.push_back(t);
-                if ((int64_t)q < f->nfallback_tiles) ++nheavy;
+                const bool heavy = (int64_t)q < f->nfallback_tiles;
+                sub.push_back(heavy ? t : (int)((int64_t)q - f->nfallback_tiles));
+                if (heavy) ++nheavy;
             }
         }
         if (!f->sub_items) FCUDA(dmalloc(&f->sub_items, sizeof(int) * std::max<int64_t>(f->nitems, 1)), "cudaMalloc");
@@ -511,17 +521,12 @@ int mlens_shoot_learned(mlens_ctx *ctx, const mlens_grid *rays, const mlens_grid
     L.plain.stats = ctx->d_stats;
     L.plain.beta_out = beta_dev;
     L.cg = f->cg;
-    L.cstart = f->start;
     L.cstars = f->cstars;
-    L.coef = f->coef;
-    L.sc = f->sc;
-    L.ec = f->ec;
-    L.params = f->params;
+    L.desc = f->desc;
+    L.cells = f->cells;
     L.w2b = f->w2b;
     L.pe = f->pe;
     L.use_net = f->use_net;
-    L.items = items;
-    L.nitems = nitems;
     L.counter = f->counter;
     L.err = f->d_err;
     L.wait_probe = g_wait_probe.load();
@@ -531,7 +536,7 @@ int mlens_shoot_learned(mlens_ctx *ctx, const mlens_grid *rays, const mlens_grid
     // time; the persistent learned kernel then takes the learned tiles.
     FCUDA(launch_shoot_split_list(L.plain, items, nheavy, fallback_star_split(ctx->n_pad), s, ctx->fma_pairs),
           "fallback tiles launch");
-    L.items = items + nheavy;
+    L.items = all_rows ? nullptr : items + nheavy;
     L.nitems = nitems - nheavy;
     if (L.nitems > 0) FCUDA(ff_shoot_learned(L, f->grid, s), "learned shoot launch");
     if (stats_host) {
@@ -685,7 +690,7 @@ int mlens_load_far_field(mlens_ctx *ctx, const char *path, void *stream)
     FCUDA(cudaMemcpy(f->flags, fl.data(), sizeof(int) * nrc, cudaMemcpyHostToDevice), "memcpy");
     FCUDA(cudaMemcpy(f->vmax_net, vn.data(), sizeof(unsigned) * nrc, cudaMemcpyHostToDevice), "memcpy");
     FCUDA(cudaMemcpy(f->vmax_series, vs.data(), sizeof(unsigned) * nrc, cudaMemcpyHostToDevice), "memcpy");
-    if ((rc = schedule(f, s))) return rc;
+    if ((rc = schedule(ctx, f, s))) return rc;
     if ((rc = finish_inference_tables(f, s))) return rc;
     FCUDA(cudaStreamSynchronize(s), "sync");
     f->ready = true;

@@ -189,13 +189,15 @@ __device__ __forceinline__ void hist_zero(uint32_t *h)
 }
 
 // Add the window to the global map (bins outside the map are never filled).
-template <int WN>
+// CLEAR: and leave it cleared for the next tile.
+template <bool CLEAR = false, int WN>
 __device__ __forceinline__ void hist_flush(const WinHist<WN> &W, const BinGrid &g, uint32_t *counts)
 {
-    const uint4 *h4 = reinterpret_cast<const uint4 *>(W.h);
+    uint4 *h4 = reinterpret_cast<uint4 *>(W.h);
     for (int b = threadIdx.x; b < WN * WN / 4; b += blockDim.x) {
         const uint4 v = h4[b];
         if ((v.x | v.y | v.z | v.w) == 0u) continue;
+        if (CLEAR) h4[b] = make_uint4(0u, 0u, 0u, 0u);
         const int64_t base = (int64_t)(W.wy0 + b / (WN / 4)) * g.nx + (W.wx0 + 4 * (b % (WN / 4)));
         if (v.x) atomicAdd(&counts[base + 0], v.x);
         if (v.y) atomicAdd(&counts[base + 1], v.y);
