@@ -326,21 +326,24 @@ __global__ void __launch_bounds__(kThr) k_disk(const int64_t *__restrict__ P, in
 // The row stride S is a template parameter, so that the rows' loads have immediate
 // addresses; S = 4 x odd, four segments of S / 4 words: the scan's 8 rows x 4 segments
 // per warp fall on 32 different banks.
-// Sums are exact in 32 bits, modulo 2^32 in the prefixes, while the largest staged count
-// times |K| is below 2^32 (`limit`; 3.2e6 rays in a pixel for 1317 pixels).  A tile with
-// larger counts takes its sums from the counts' low and high halves in two passes per eight
-// rows, in 64 bits.
-// Bound by shared-memory loads, 59 of 4 bytes per output at R = 20 pixels: 4096^2 pixels in
-// 164 us, 373 us with int64 prefixes made by a kernel of their own and staged with their
-// halo (8 bytes a load, and three FP64 operations per output); R = 45 1959 -> 456 us.
+// Where every staged row's total fits 13 bits the prefixes are kept as 16-bit numbers, two
+// neighbouring ones a word, and a thread sums two columns at once (disk_sums): half the
+// loads and additions.  Elsewhere sums are exact in 32 bits, modulo 2^32 in the prefixes,
+// while the largest staged count times |K| is below 2^32 (`limit`; 3.2e6 rays in a pixel for
+// 1317 pixels).  A tile with larger counts takes its sums from the counts' low and high halves
+// in two passes per eight rows, in 64 bits.
+// Bound by issue slots (77 %) and shared-memory loads (30 words an output at R = 20 pixels
+// packed, 59 not): 4096^2 pixels in 130 us; 164 us unpacked; 373 us with int64 prefixes made
+// by a kernel of their own and staged with their halo (8 bytes a load, three FP64 operations
+// per output).  R = 45 1959 -> 316 us, R = 79 2788 -> 871 us.
 constexpr int kMaxGroups = 256;  // runs of support rows of one half-width that a plan carries
 struct DiskGroups {
     int n;
     uint16_t half[kMaxGroups], rows[kMaxGroups];
 };
 
-// The groups cut into blocks of 8, 4, 2 and 1 rows (integer sums take any order), each the
-// stage offsets of its first row's upper and lower prefix value; passed by value with
+// The groups cut into blocks of 8, 4, 2 and 1 rows (integer sums take any order): the
+// stage offset of a block's first row and its half-width; passed by value with
 // the launch and read from the constant bank.
 constexpr int kMaxBlocks = 384;
 struct DiskBlocks {
@@ -375,19 +378,109 @@ __device__ __forceinline__ float scale_sum(uint32_t s, double f, float fh, float
     return scale_sum_fp64(s, f);
 }
 
+// Sums of R output rows of one staged column (PACKED: of two adjacent ones, in the halves
+// of a word) over the support's blocks.  base: the column in the first of the rows.
+// PACKED words hold two neighbouring prefix values each, in two copies of a row: word k of
+// the first S / 2 is (P[2k], P[2k+1]), of the others (P[2k+1], P[2k+2]), so that a pair of
+// columns reads one word at any offset.  The prefixes do not decrease and are below 2^16, so
+// a word's difference is both columns' runs; `room` rows of runs fit a half, then the sums
+// move to lo and hi.
+template <int S, int W, int R, bool PACKED>
+__device__ __forceinline__ void disk_sums(const uint32_t *base, const DiskBlocks &B, int room, uint32_t (&sum)[R],
+                                          uint32_t (&lo_s)[R], uint32_t (&hi_s)[R])
+{
+#pragma unroll
+    for (int k = 0; k < R; ++k) sum[k] = lo_s[k] = hi_s[k] = 0;
+    const uint32_t *hi = nullptr, *lo = nullptr;
+    auto run = [&](int q) { return hi[q * S] - lo[q * S]; };  // row q of the block
+    auto at = [&](int n) {
+        const int2 e = B.at[n];
+        const int xh = W + 1 + e.y, xl = W - e.y;
+        hi = base + e.x + (PACKED ? (xh >> 1) + (xh & 1) * (S / 2) : xh);
+        lo = base + e.x + (PACKED ? (xl >> 1) + (xl & 1) * (S / 2) : xl);
+    };
+    int left = room;
+    auto make_room = [&](int m) {
+        if (!PACKED) return;
+        if (left < m) {
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                lo_s[k] += sum[k] & 0xffffu;
+                hi_s[k] += sum[k] >> 16;
+                sum[k] = 0;
+            }
+            left = room;
+        }
+        left -= m;
+    };
+    int n = 0;
+    for (; n < B.n8; ++n) {
+        at(n);
+        make_room(8);
+        uint32_t r[R + 7];
+#pragma unroll
+        for (int q = 0; q < R + 7; ++q) r[q] = run(q);
+#pragma unroll
+        for (int q = 0; q < R + 6; ++q) r[q] += r[q + 1];
+#pragma unroll
+        for (int q = 0; q < R + 4; ++q) r[q] += r[q + 2];
+#pragma unroll
+        for (int k = 0; k < R; ++k) sum[k] += r[k] + r[k + 4];
+    }
+    for (; n < B.n4; ++n) {
+        at(n);
+        make_room(4);
+        uint32_t r[R + 3];
+#pragma unroll
+        for (int q = 0; q < R + 3; ++q) r[q] = run(q);
+#pragma unroll
+        for (int q = 0; q < R + 2; ++q) r[q] += r[q + 1];
+#pragma unroll
+        for (int k = 0; k < R; ++k) sum[k] += r[k] + r[k + 2];
+    }
+    for (; n < B.n2; ++n) {
+        at(n);
+        make_room(2);
+        uint32_t r[R + 1];
+#pragma unroll
+        for (int q = 0; q < R + 1; ++q) r[q] = run(q);
+#pragma unroll
+        for (int k = 0; k < R; ++k) sum[k] += r[k] + r[k + 1];
+    }
+#pragma unroll 2
+    for (; n < B.n1; ++n) {
+        at(n);
+        make_room(1);
+#pragma unroll
+        for (int k = 0; k < R; ++k) sum[k] += run(k);
+    }
+    if (PACKED) {
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            lo_s[k] += sum[k] & 0xffffu;
+            hi_s[k] += sum[k] >> 16;
+        }
+    }
+}
+
 template <int TX, int TY, int S>
 __global__ void __launch_bounds__(kThr) k_disk_tile(const uint32_t *__restrict__ in, int nx, int ny,
                                                     const __grid_constant__ DiskBlocks B, int H, uint32_t limit,
                                                     double f, float fh, float fl, bool fast, float *__restrict__ out)
 {
     extern __shared__ __align__(16) uint32_t T[];
+    __shared__ uint32_t s_top, s_row;  // the largest staged count and row total
     constexpr int kGroup = kThr / TX, kRows = 8, kPer = TY / kGroup;  // output rows per thread, kRows at a time
-    static_assert(kThr % TX == 0 && kPer % kRows == 0, "whole batches");
+    constexpr int kSeg = S / 4;
+    // packed pairs of columns: the segment of a scan is held in registers
+    constexpr bool kPacks = kSeg <= 51;
+    constexpr int kGroup2 = 2 * kGroup, kPer2 = TY / kGroup2, kRows2 = kPer2 < 8 ? kPer2 : 8;
+    static_assert(kThr % TX == 0 && kPer % kRows == 0 && kPer2 % kRows2 == 0, "whole batches");
     static_assert(S % 8 == 4, "conflict-free scan");
     constexpr int W = disk_tile_w(TX, S);  // the staged columns start at i0 - W - 1
     const int rows = TY + 2 * H;
-    const int tid = threadIdx.x, c = tid % TX, g = tid / TX;
-    const int i0 = blockIdx.x * TX, i = i0 + c;
+    const int tid = threadIdx.x;
+    const int i0 = blockIdx.x * TX;
     const int64_t tiles_y = ((int64_t)ny + TY - 1) / TY;
     for (int64_t by = blockIdx.y; by < tiles_y; by += gridDim.y) {
         const int64_t j0 = by * TY;
@@ -407,19 +500,19 @@ __global__ void __launch_bounds__(kThr) k_disk_tile(const uint32_t *__restrict__
             cp_async_wait_all();
             __syncthreads();
         };
-        // rows to prefix sums of (count >> shift) & mask, four lanes per row; returns the largest count seen
+        // rows to prefix sums of (count >> shift) & mask, four lanes per row; the largest
+        // count seen to s_top
         auto scan = [&](int shift, uint32_t mask) {
             uint32_t top = 0;
             for (int base = 0; base < rows; base += kThr / 4) {
                 const int r = base + tid / 4;
-                uint32_t *p = T + r * S + (tid & 3) * (S / 4);
+                uint32_t *p = T + r * S + (tid & 3) * kSeg;
                 uint32_t sum = 0;
                 if (r < rows) {
 #pragma unroll 8
-                    for (int k = 0; k < S / 4; ++k) {
-                        const uint32_t v = p[k];
-                        top = max(top, v);
-                        sum += (v >> shift) & mask;
+                    for (int k = 0; k < kSeg; ++k) {
+                        top = max(top, p[k]);
+                        sum += (p[k] >> shift) & mask;
                     }
                 }
                 uint32_t inc = sum;  // inclusive over the row's four lanes
@@ -431,92 +524,126 @@ __global__ void __launch_bounds__(kThr) k_disk_tile(const uint32_t *__restrict__
                 uint32_t run = inc - sum;
                 if (r < rows) {
 #pragma unroll 8
-                    for (int k = 0; k < S / 4; ++k) {
+                    for (int k = 0; k < kSeg; ++k) {
                         run += (p[k] >> shift) & mask;
                         p[k] = run;
                     }
                 }
             }
-            return top;
+            top = __reduce_max_sync(0xffffffffu, top);
+            if ((tid & 31) == 0) atomicMax(&s_top, top);
+            __syncthreads();
         };
-        // sums of the batch of eight rows from output row rt on
-        auto sums = [&](int rt, uint32_t (&sum)[kRows]) {
-            // row rt + d of the stage is row j0 + rt - H + d of the map; tr[0] is the column of i
-            const uint32_t *tr = T + rt * S + c + W;
+        // rows to packed prefix sums, in place: a row's four lanes (one warp) have read it
+        // before they write
+        auto scan_packed = [&]() {
+            for (int base = 0; base < rows; base += kThr / 4) {
+                const int r = base + tid / 4, seg = tid & 3;
+                uint32_t *row = T + r * S;
+                uint32_t v[kSeg + 1], sum = 0;
 #pragma unroll
-            for (int k = 0; k < kRows; ++k) sum[k] = 0;
-            int n = 0;
-            // run sum of row q of a block; a block of M rows adds run(k) + .. + run(k + M - 1) to output k
-            const uint32_t *hi, *lo;
-            auto run = [&](int q) { return hi[q * S] - lo[q * S]; };
-            for (; n < B.n8; ++n) {
-                hi = tr + B.at[n].x, lo = tr + B.at[n].y;
-                uint32_t r[kRows + 7];
-#pragma unroll
-                for (int q = 0; q < kRows + 7; ++q) r[q] = run(q);
-#pragma unroll
-                for (int q = 0; q < kRows + 6; ++q) r[q] += r[q + 1];
-#pragma unroll
-                for (int q = 0; q < kRows + 4; ++q) r[q] += r[q + 2];
-#pragma unroll
-                for (int k = 0; k < kRows; ++k) sum[k] += r[k] + r[k + 4];
-            }
-            for (; n < B.n4; ++n) {
-                hi = tr + B.at[n].x, lo = tr + B.at[n].y;
-                uint32_t r[kRows + 3];
-#pragma unroll
-                for (int q = 0; q < kRows + 3; ++q) r[q] = run(q);
-#pragma unroll
-                for (int q = 0; q < kRows + 2; ++q) r[q] += r[q + 1];
-#pragma unroll
-                for (int k = 0; k < kRows; ++k) sum[k] += r[k] + r[k + 2];
-            }
-            for (; n < B.n2; ++n) {
-                hi = tr + B.at[n].x, lo = tr + B.at[n].y;
-                uint32_t r[kRows + 1];
-#pragma unroll
-                for (int q = 0; q < kRows + 1; ++q) r[q] = run(q);
-#pragma unroll
-                for (int k = 0; k < kRows; ++k) sum[k] += r[k] + r[k + 1];
-            }
-#pragma unroll 2
-            for (; n < B.n1; ++n) {
-                hi = tr + B.at[n].x, lo = tr + B.at[n].y;
-#pragma unroll
-                for (int k = 0; k < kRows; ++k) sum[k] += run(k);
-            }
-        };
-        stage();
-        const uint32_t top = scan(0, 0xffffffffu);
-        const bool large = __syncthreads_or(top > limit);
-        for (int b = 0; b < kPer; b += kRows) {
-            const int rt = g * kPer + b;
-            uint32_t sum[kRows];
-            if (!large) {
-                if (i < nx && j0 + rt < ny) {
-                    sums(rt, sum);
-#pragma unroll
-                    for (int k = 0; k < kRows; ++k)
-                        if (j0 + rt + k < ny) out[(j0 + rt + k) * nx + i] = scale_sum(sum[k], f, fh, fl, fast);
+                for (int k = 0; k < kSeg; ++k) {
+                    v[k] = r < rows ? row[seg * kSeg + k] : 0u;
+                    sum += v[k];
                 }
-            } else {
-                uint32_t hi[kRows];
-                stage();
-                scan(0, 0xffffu);
-                __syncthreads();
-                sums(rt, sum);
-                stage();
-                scan(16, 0xffffu);
-                __syncthreads();
-                sums(rt, hi);
+                uint32_t inc = sum;
 #pragma unroll
-                for (int k = 0; k < kRows; ++k)
-                    if (i < nx && j0 + rt + k < ny) {
-                        const int64_t s = (int64_t)sum[k] + ((int64_t)hi[k] << 16);
-                        out[(j0 + rt + k) * nx + i] = __double2float_rn(__dmul_rn((double)s, f));
+                for (int d = 1; d < 4; d <<= 1) {
+                    const uint32_t o = __shfl_up_sync(0xffffffffu, inc, d, 4);
+                    if (seg >= d) inc += o;
+                }
+                v[kSeg] = __shfl_down_sync(0xffffffffu, v[0], 1, 4);  // the next segment's first (unread behind the last)
+                __syncwarp();
+                if (r < rows) {
+                    uint32_t run = inc - sum + v[0];  // P at the segment's first element
+                    const int odd = (seg * kSeg) & 1;
+                    uint32_t *even_w = row + (seg * kSeg + odd) / 2, *odd_w = row + S / 2 + (seg * kSeg - odd) / 2;
+                    // element g = seg kSeg + k goes, with its successor, to word g / 2 of the even or the odd copy
+#pragma unroll
+                    for (int k = 0; k < kSeg; ++k) {
+                        const uint32_t nxt = run + v[k + 1], w = run | nxt << 16;
+                        if (((k ^ odd) & 1) == 0)
+                            even_w[(k - odd + (k & 1)) / 2] = w;
+                        else
+                            odd_w[(k + odd - (odd ? 0 : 1)) / 2] = w;
+                        run = nxt;
+                    }
+                }
+            }
+            __syncthreads();
+        };
+        if (tid == 0) s_top = s_row = 0u;
+        stage();
+        uint32_t most = 0xffffffffu;
+        if (kPacks) {  // the largest row total (counts saturate at 16 bits: it is only compared with 8191)
+            most = 0;
+            for (int base = 0; base < rows; base += kThr / 4) {
+                const int r = base + tid / 4;
+                const uint32_t *p = T + r * S + (tid & 3) * kSeg;
+                uint32_t sum = 0;
+                if (r < rows) {
+#pragma unroll 8
+                    for (int k = 0; k < kSeg; ++k) sum += min(p[k], 0xffffu);
+                }
+                sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+                sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+                most = max(most, sum);
+            }
+            most = __reduce_max_sync(0xffffffffu, most);
+            if ((tid & 31) == 0) atomicMax(&s_row, most);
+            __syncthreads();
+            most = s_row;
+        }
+        if (kPacks && most <= 8191u) {
+            // eight rows of runs fit 16 bits (with one count above 0xffff the total is above too)
+            scan_packed();
+            const int c = 2 * (tid % (TX / 2)), g = tid / (TX / 2), i = i0 + c;
+            const int room = (int)min(65535u / max(most, 1u), 1u << 20);
+            for (int b = 0; b < kPer2; b += kRows2) {
+                const int rt = g * kPer2 + b;
+                if (i >= nx || j0 + rt >= ny) break;
+                uint32_t sum[kRows2], lo[kRows2], hi[kRows2];
+                disk_sums<S, W, kRows2, true>(T + rt * S + c / 2, B, room, sum, lo, hi);
+#pragma unroll
+                for (int k = 0; k < kRows2; ++k)
+                    if (j0 + rt + k < ny) {
+                        float *dst = out + (j0 + rt + k) * nx + i;
+                        dst[0] = scale_sum(lo[k], f, fh, fl, fast);
+                        if (i + 1 < nx) dst[1] = scale_sum(hi[k], f, fh, fl, fast);
                     }
             }
+        } else {
+            const int c = tid % TX, g = tid / TX, i = i0 + c;
+            scan(0, 0xffffffffu);
+            const bool large = s_top > limit;
+            for (int b = 0; b < kPer; b += kRows) {
+                const int rt = g * kPer + b;
+                uint32_t sum[kRows], lo[kRows], hi[kRows];
+                if (!large) {
+                    if (i < nx && j0 + rt < ny) {
+                        disk_sums<S, W, kRows, false>(T + rt * S + c, B, 0, sum, lo, hi);
+#pragma unroll
+                        for (int k = 0; k < kRows; ++k)
+                            if (j0 + rt + k < ny) out[(j0 + rt + k) * nx + i] = scale_sum(sum[k], f, fh, fl, fast);
+                    }
+                } else {
+                    uint32_t high[kRows];
+                    stage();
+                    scan(0, 0xffffu);
+                    disk_sums<S, W, kRows, false>(T + rt * S + c, B, 0, sum, lo, hi);
+                    stage();
+                    scan(16, 0xffffu);
+                    disk_sums<S, W, kRows, false>(T + rt * S + c, B, 0, high, lo, hi);
+#pragma unroll
+                    for (int k = 0; k < kRows; ++k)
+                        if (i < nx && j0 + rt + k < ny) {
+                            const int64_t t = (int64_t)sum[k] + ((int64_t)high[k] << 16);
+                            out[(j0 + rt + k) * nx + i] = __double2float_rn(__dmul_rn((double)t, f));
+                        }
+                }
+            }
         }
+        __syncthreads();  // s_top and s_row are set again
     }
 }
 
@@ -791,7 +918,7 @@ cudaError_t launch_disk_tile(const uint32_t *in, int nx, int ny, const ConvPlan 
             for (int q = 0; q < k; ++q) {
                 if (n == kMaxBlocks) return cudaErrorInvalidValue;  // the plan has at most kMaxGroups groups: unreachable
                 const int r = (row + r0 + q * m) * S;
-                B.at[n++] = make_int2(r + h + 1, r - h);
+                B.at[n++] = make_int2(r, h);
             }
         }
         *end[kind] = n;
@@ -805,8 +932,8 @@ cudaError_t launch_disk_tile(const uint32_t *in, int nx, int ny, const ConvPlan 
 }
 
 // The disk in one kernel: 128 x 64 outputs (the least halo) where three CTAs fit an SM
-// and the tiles fill the SMs twice, else 64 x 32; the smallest row stride with room for
-// the support.  *done = false: no tile fits its shared memory.
+// and the tiles fill the SMs twice, else 64 x 64 where they fill them once, else 64 x 32; the
+// smallest row stride with room for the support.  *done = false: no tile fits its shared memory.
 template <int TX, int TY, int S, int... More>
 cudaError_t disk_tile_of(const uint32_t *in, int nx, int ny, const ConvPlan &pl, double f, float *out, cudaStream_t s,
                          size_t most, bool *done)
@@ -850,6 +977,9 @@ int run_convolution(const uint32_t *counts_dev, const mlens_grid *src, int32_t p
         bool done = false;
         if ((int64_t)((nx + 127) / 128) * ((ny + 63) / 64) >= 2 * (int64_t)nsm)
             e = disk_tile_of<128, 64, 140, 172, 204>(counts_dev, nx, ny, pl, f, out_dev, s, kDiskTileSmem3, &done);
+        if (e == cudaSuccess && !done && (int64_t)((nx + 63) / 64) * ((ny + 63) / 64) >= (int64_t)nsm)
+            e = disk_tile_of<64, 64, 76, 108, 140, 172, 236, 300>(counts_dev, nx, ny, pl, f, out_dev, s, kDiskTileSmem1,
+                                                                  &done);
         if (e == cudaSuccess && !done)
             e = disk_tile_of<64, 32, 76, 108, 140, 172, 236, 300>(counts_dev, nx, ny, pl, f, out_dev, s, kDiskTileSmem1,
                                                                   &done);

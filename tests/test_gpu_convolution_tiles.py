@@ -79,3 +79,20 @@ def test_gaussian_at_width_and_tap_edges(nx, px):
     # 2 Kx + 1 and 2 Ky + 1 products and sums of non-negative terms, weights and scale rounded
     bound = 2.0 * (2 * kx + 2 * ky + 8) * 2.0 ** -24 * np.abs(ref) + 1e-30
     assert np.all(np.abs(got[js, is_] - ref) <= bound)
+
+
+@pytest.mark.parametrize("px", [3.2, 21.6, 37.4, 53.2, 80.0])
+@pytest.mark.parametrize("mean", [6.0, 40.0, 60.0])
+def test_disk_square_tiles_and_packed_sums(px, mean):
+    """A map of enough 64 x 64 tiles but not enough 128 x 64 ones; mean counts whose row totals
+    fit 16 bits with room for all rows of the support, with room for a few, and not at all."""
+    rng = np.random.default_rng(int(px + mean))
+    nx, ny = 1025, 701
+    src = W.Grid(0.0, nx * 0.01, 0.0, ny * 0.01, nx, ny)
+    c = rng.poisson(mean, (ny, nx)).astype(np.uint32)
+    c[300:400, 100:900:7] = int(20 * mean)  # some tiles beyond, their neighbours within
+    got = _conv(c, src, M.MLENS_PROFILE_DISK, px * 0.01, 0.7)
+    js, is_ = rng.integers(0, ny, 120), rng.integers(0, nx, 120)
+    js[:4], is_[:4] = (0, 0, ny - 1, ny - 1), (0, nx - 1, 0, nx - 1)
+    ref = LC.convolve_at(c, src, LC.DISK, px * 0.01, 0.7, js, is_).astype(np.float32)
+    assert np.array_equal(got[js, is_].view(np.uint32), ref.view(np.uint32))
