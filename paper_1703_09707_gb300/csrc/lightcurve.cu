@@ -86,13 +86,16 @@ __device__ __forceinline__ void gauss_step(float2 (&acc)[N], const float2 (&x)[N
 // loads of element 8t + k are consecutive.  TX follows the map's width (run_convolution):
 // 1024 outputs per row pair need the least halo, narrower maps would leave threads
 // without outputs.
-// Bound by the FP32 pipe and the staging's latency: 83 taps over 4096^2 pixels 83 ->
-// 71 us (the multiply-adds alone take 35 us); the whole call 182 -> 131 us, 300 x 2000
-// pixels and 97 taps 37 -> 21 us.
+// Where rows start on 16 bytes a thread stores its outputs itself, as two float4 a row;
+// else they go through the planes, so that the lanes store consecutive pixels.
+// Bound by the FP32 pipe and the staging's latency: 83 taps over 4096^2 pixels 83 -> 61
+// us (the multiply-adds alone take 35 us); the whole call 182 -> 119 us.
+// Five CTAs an SM and three elements in flight: against 121 us in one timing, four or six
+// CTAs 126, two or five elements 134 and 130, all outputs through the planes 126 us.
 template <int TX>
-__global__ void __launch_bounds__(kThr) k_gauss_rows(const uint32_t *__restrict__ in, int nx, int ny,
-                                                     const __grid_constant__ GaussTaps W, int K,
-                                                     float *__restrict__ out)
+__global__ void __launch_bounds__(kThr, 5) k_gauss_rows(const uint32_t *__restrict__ in, int nx, int ny,
+                                                        const __grid_constant__ GaussTaps W, int K,
+                                                        float *__restrict__ out)
 {
     extern __shared__ float2 sm2[];
     const int Kp = taps_padded(K);
@@ -107,7 +110,7 @@ __global__ void __launch_bounds__(kThr) k_gauss_rows(const uint32_t *__restrict_
         const bool one = j < ny, two = j + 1 < ny;
         const uint32_t *row0 = in + j * nx, *row1 = row0 + nx;
         __syncthreads();  // previous rows' taps are done
-        constexpr int kB = 5;  // elements of each row in flight per thread
+        constexpr int kB = 3;  // elements of each row in flight per thread
         for (int e0 = t; e0 < E; e0 += kB * TX) {
             uint32_t v0[kB], v1[kB];
 #pragma unroll
@@ -150,6 +153,20 @@ __global__ void __launch_bounds__(kThr) k_gauss_rows(const uint32_t *__restrict_
                 step(m + 4, 1);
             }
             if (m < Kp) step(m, 0);
+        }
+        if (nx % 4 == 0) {  // of a thread's two groups of four outputs the first is in the row, the second may not be
+            if (o < nx && one) {
+                float4 *d = reinterpret_cast<float4 *>(out + j * nx + o);
+                const bool both = o + 4 < nx;
+                d[0] = make_float4(acc[0].x, acc[1].x, acc[2].x, acc[3].x);
+                if (both) d[1] = make_float4(acc[4].x, acc[5].x, acc[6].x, acc[7].x);
+                if (two) {
+                    d += nx / 4;
+                    d[0] = make_float4(acc[0].y, acc[1].y, acc[2].y, acc[3].y);
+                    if (both) d[1] = make_float4(acc[4].y, acc[5].y, acc[6].y, acc[7].y);
+                }
+            }
+            continue;
         }
         // outputs through the planes, so that the lanes store consecutive pixels (a
         // thread's own eight would touch a sector per lane and store)

@@ -96,3 +96,21 @@ def test_disk_square_tiles_and_packed_sums(px, mean):
     js[:4], is_[:4] = (0, 0, ny - 1, ny - 1), (0, nx - 1, 0, nx - 1)
     ref = LC.convolve_at(c, src, LC.DISK, px * 0.01, 0.7, js, is_).astype(np.float32)
     assert np.array_equal(got[js, is_].view(np.uint32), ref.view(np.uint32))
+
+
+@pytest.mark.parametrize("nx,ny", [(4, 1), (12, 33), (252, 17), (260, 16), (508, 7), (516, 9), (1028, 5), (2052, 3)])
+@pytest.mark.parametrize("px", [1.0, 30.3])
+def test_gaussian_rows_of_whole_vectors(nx, ny, px):
+    """Widths of whole float4 whose last thread has one of its two; odd row counts; every row
+    checked at both ends."""
+    rng = np.random.default_rng(nx + ny)
+    src = W.Grid(0.0, nx * 0.01, 0.0, ny * 0.01, nx, ny)
+    c = _counts(rng, ny, nx, "spikes")
+    got = _conv(c, src, M.MLENS_PROFILE_GAUSSIAN, px * 0.01, 0.37)
+    edges = np.unique(np.r_[:min(nx, 9), max(nx - 9, 0):nx])
+    js, is_ = (v.ravel() for v in np.meshgrid(np.arange(ny), edges, indexing="ij"))
+    ref = LC.convolve_at(c, src, LC.GAUSSIAN, px * 0.01, 0.37, js, is_)
+    k = math.ceil(4 * px)
+    # 2 k + 1 products and sums of non-negative terms per pass, weights and scale rounded
+    bound = 2.0 * (4 * k + 8) * 2.0 ** -24 * np.abs(ref) + 1e-30
+    assert np.all(np.abs(got[js, is_] - ref) <= bound)
