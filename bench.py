@@ -809,7 +809,7 @@ def run_mine(args):
         "maps_per_s": args.steps * (1 if strong else world) / dev_s,
         "roofline": roof,
         "e2e": e2e,
-        "gpu_launches": args.steps,
+        "gpu_launches": 2 * args.steps,  # a shot is the clears' launch and the sum's
         "clocks": clk,
         "wall_s_timed": t_wall,
         "device": props.name,

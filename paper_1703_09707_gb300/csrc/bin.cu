@@ -9,12 +9,13 @@
 // records of one grid row would instead spread along a strip of the map far longer
 // than the window).
 //
-// Bound by HBM in grid order: 8192^2 records (1.07 GB) into 1024^2 pixels in 0.164 ms
-// = 6.6 TB/s, 0.97 of the measured copy rate; 0.292 ms, bound by its 114 instructions a
-// record, before the fast pixel rule (mlens_dev.cuh).  Flat order 0.271 -> 0.214 ms,
-// bound by the global atomics of records outside the window.  Four records in flight
-// per thread and eight CTAs of 32 registers per SM: eight records and four CTAs
-// 0.181 ms, eight and five 0.170, sixteen and three 0.210; 8192 records per CTA 0.167.
+// Bound by HBM in grid order: 8192^2 records (1.07 GB) into 1024^2 pixels in 0.160 ms
+// = 6.7 TB/s, 0.99 of the measured copy rate; 0.292 ms, bound by its 114 instructions a
+// record, before the fast pixel rule (mlens_dev.cuh), 0.164 before the clears ran
+// alongside the first loads (clear.cu).  Flat order 0.271 -> 0.214 ms, bound by the global
+// atomics of records outside the window.  Four records in flight per thread and eight
+// CTAs of 32 registers per SM; against 0.164: eight records and four CTAs 0.181 ms, eight
+// and five 0.170, sixteen and three 0.210; 8192 records per CTA 0.167.
 #include <cuda_runtime.h>
 #include <stdint.h>
 

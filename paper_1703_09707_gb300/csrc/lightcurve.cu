@@ -32,6 +32,7 @@ namespace mlens {
 namespace {
 
 constexpr int kThr = 256;
+constexpr size_t kConvSmemMost = 226 * 1024;  // above every convolution kernel's dynamic shared memory
 constexpr int kColX = 64;       // column pass: tile columns
 constexpr int kColY = 128;      // column pass: tile rows
 constexpr int kMaxTaps = 256;   // Gaussian half-width limit (pixels)
@@ -896,7 +897,7 @@ cudaError_t launch_gauss_rows(const uint32_t *in, int nx, int ny, const GaussTap
 {
     constexpr int kPairs = kThr / TX;
     const size_t smem = (size_t)kPairs * 8 * ((8 * TX + taps_padded(K) + 7) / 8 + 1) * sizeof(float2);
-    const cudaError_t e = allow_dynamic_smem(k_gauss_rows<TX>, smem);
+    const cudaError_t e = allow_dynamic_smem(k_gauss_rows<TX>, smem, kConvSmemMost);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)((nx + 8 * TX - 1) / (8 * TX)),
                     (unsigned)std::min<int64_t>((ny + 2 * kPairs - 1) / (2 * kPairs), 65535));
@@ -909,7 +910,7 @@ cudaError_t launch_gauss_cols(const float *in, int nx, int ny, const GaussTaps &
                               cudaStream_t s)
 {
     const size_t smem = (size_t)(kColY + taps_padded(K) + 3) * kColX * sizeof(float);
-    const cudaError_t e = allow_dynamic_smem(k_gauss_cols<VEC>, smem);
+    const cudaError_t e = allow_dynamic_smem(k_gauss_cols<VEC>, smem, kConvSmemMost);
     if (e != cudaSuccess) return e;
     const int64_t tiles_y = (ny + kColY - 1) / kColY;
     const dim3 grid((unsigned)((nx + kColX - 1) / kColX), (unsigned)std::min<int64_t>(tiles_y, 65535));
@@ -922,7 +923,7 @@ cudaError_t launch_disk_tile(const uint32_t *in, int nx, int ny, const ConvPlan 
                              cudaStream_t s)
 {
     const size_t smem = (size_t)(TY + 2 * pl.Hs) * S * sizeof(uint32_t);
-    const cudaError_t e = allow_dynamic_smem(k_disk_tile<TX, TY, S>, smem);
+    const cudaError_t e = allow_dynamic_smem(k_disk_tile<TX, TY, S>, smem, kConvSmemMost);
     if (e != cudaSuccess) return e;
     DiskBlocks B{};
     int n = 0, *end[4] = {&B.n8, &B.n4, &B.n2, &B.n1};

@@ -95,11 +95,14 @@ struct BatchLaunch {
 };
 
 // Let a kernel take `bytes` of dynamic shared memory, with the largest shared-memory
-// carveout of the SM (two CTAs of up to ~110 KB).
+// carveout of the SM.  The limit belongs to the kernel, not to the call: a kernel whose size
+// varies names its `most`, always set, so that a second thread's smaller call cannot
+// lower the limit between this thread's setting and its launch.
 template <class K>
-inline cudaError_t allow_dynamic_smem(K kernel, size_t bytes)
+inline cudaError_t allow_dynamic_smem(K kernel, size_t bytes, size_t most = 0)
 {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(bytes > most ? bytes : most));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                  (int)cudaSharedmemCarveoutMaxShared);

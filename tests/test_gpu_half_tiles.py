@@ -86,3 +86,24 @@ def test_captured_calls_replay():
             assert np.array_equal(c.cpu().numpy().view(np.uint32).reshape(src.ny, src.nx), want)
         assert np.array_equal(beta.cpu().numpy().view(np.uint32), b4.reshape(-1).view(np.uint32))
     ctx.close()
+
+
+@pytest.mark.parametrize("blocks", [1, 4, 5, 8, 9, 12, 13])
+@pytest.mark.parametrize("rpt,precision", [(8, "fp32"), (4, "fp32"), (8, "fp32_naive")])
+def test_grids_of_few_ctas_equal_their_bands(blocks, rpt, precision):
+    """38 half tiles per 32 rows: up to one, two, three or more CTAs on each of 152 SMs, and
+    every band of 32 rows, launched with at most one per SM, gives the same positions and map."""
+    f = W.random_field(W.SEED_BASE + 700, 300, kappa_star=0.35, kappa_c=0.1, gamma1=0.2, gamma2=0.07)
+    ny = 32 * blocks - (5 if blocks > 1 else 0)
+    rays, src = W.Grid(-3.0, 3.0, -2.0, 2.0, 1200, ny), W.Grid(-2.0, 2.0, -2.0, 2.0, 90, 40)
+    ctx = M.mlens_create(f.xy, f.m, f.kappa_c, f.gamma1, f.gamma2, precision)
+    M.mlens_set_tuning(ctx, rpt)
+    M.mlens_set_star_split(ctx, 1)
+    whole, bands = (torch.zeros((40, 90), dtype=torch.int32, device="cuda") for _ in range(2))
+    b0, b1 = (torch.zeros((ny, 1200, 4), dtype=torch.float32, device="cuda") for _ in range(2))
+    M.mlens_shoot_beta(ctx, rays, src, whole, b0)
+    for r in range(0, ny, 32):
+        M.mlens_shoot_rows(ctx, rays, (r, min(r + 32, ny)), src, bands, beta=b1, flags=M.MLENS_ACCUMULATE)
+    ctx.close()
+    assert whole.any() and torch.equal(whole, bands)
+    assert torch.equal(b0.view(torch.int32), b1.view(torch.int32))
