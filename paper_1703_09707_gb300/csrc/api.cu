@@ -137,9 +137,10 @@ int read_stats(unsigned long long *d_stats, uint64_t total, mlens_stats *st, cud
 
 // The map (unless the call accumulates) and the three ray counters to zero, one launch.
 cudaError_t clear_map(uint32_t *counts, const mlens_grid *src, uint32_t flags, unsigned long long *stats,
-                      cudaStream_t s)
+                      cudaStream_t s, int carveout = (int)cudaSharedmemCarveoutMaxShared)
 {
     ClearArgs c{};
+    c.carveout = carveout;
     c.map = counts;
     c.n = flags & MLENS_ACCUMULATE ? 0 : (size_t)src->nx * (size_t)src->ny;
     c.words[0] = reinterpret_cast<uint32_t *>(stats);
@@ -386,7 +387,7 @@ int bin_impl(const void *beta_dev, int64_t n, int rnx, int rny, const mlens_grid
     unsigned long long *st = nullptr;
     if ((rc = device_scratch(&st))) return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    MLENS_CUDA(clear_map(counts_dev, src, flags, st, s), "clear launch");
+    MLENS_CUDA(clear_map(counts_dev, src, flags, st, s, bin_clear_carveout(n)), "clear launch");
     BinArgs a{};
     a.beta = reinterpret_cast<const float4 *>(beta_dev);
     a.n = n;

@@ -88,6 +88,22 @@ __device__ __forceinline__ void bin_block(const BinArgs &a)
 __global__ void __launch_bounds__(kBinThreads, 8) k_bin_grid(BinArgs a) { bin_block<true>(a); }
 __global__ void __launch_bounds__(kBinThreads, 8) k_bin_flat(BinArgs a) { bin_block<false>(a); }
 
+// 72 %: eight CTAs of a 16 KB window and 1 KB reserved, 137 of 228 KB, in the next size there
+// is.  2^16 random records into 4096^2 pixels 29.8 -> 15.4 us (with the clear and the kernel
+// one after the other 16.0), 500^2 rays in order 23.6 -> 16.1 us.  Below four CTAs per SM;
+// more fill the chip however they are placed, and then do better behind any clear: 2^22
+// records into 2900^2 pixels 31 us, 33 us behind the same carveout, 8192^2 rays into 1024^2 pixels
+// 158.8 and 160.1 us.  (The largest carveout spreads them too, but leaves the kernel little L1:
+// 8192^2 rays into 4096^2 pixels 224 -> 238 us.)
+int bin_clear_carveout(int64_t n)
+{
+    int dev = 0, nsm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return -1;
+    return n <= (int64_t)kBinRecs * 4 * nsm ? 72 : -1;
+}
+
 cudaError_t launch_bin(const BinArgs &a, cudaStream_t s)
 {
     if (a.n <= 0) return cudaSuccess;

@@ -4,6 +4,9 @@
 // neither, and waits for the clears (pdl_wait) before its first increment.  Two or
 // four cudaMemsetAsync, each a node of its own before the kernel could start, took 3 us of
 // a 49 us map (100 stars, 1000^2 rays) and 4 us of binning 8192^2 records (163 -> 159 us).
+// The clear takes the shared-memory carveout of the kernel behind it although it uses no
+// shared memory: an SM takes no CTA that needs another carveout before it has drained, so that
+// kernel's first CTAs would crowd on the few SMs that drain first.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -31,8 +34,16 @@ __global__ void __launch_bounds__(256) k_clear(ClearArgs a)
 cudaError_t launch_clear(const ClearArgs &a, cudaStream_t s)
 {
     const size_t blocks = std::min<size_t>((a.n / 4 + 255) / 256 + 1, 2048);
-    k_clear<<<(unsigned)blocks, 256, 0, s>>>(a);
-    return cudaGetLastError();
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[0].val.sharedMemCarveout = (unsigned)a.carveout;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3(256);
+    cfg.stream = s;
+    cfg.attrs = attr;
+    cfg.numAttrs = a.carveout < 0 ? 0 : 1;
+    return cudaLaunchKernelEx(&cfg, k_clear, a);
 }
 
 }  // namespace mlens

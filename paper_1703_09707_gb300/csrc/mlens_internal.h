@@ -112,6 +112,7 @@ inline cudaError_t allow_dynamic_smem(K kernel, size_t bytes, size_t most = 0)
 // Zero words before a call's kernel (clear.cu): a map of n words (n = 0: none) and up
 // to three short runs of words.
 struct ClearArgs {
+    int carveout = (int)cudaSharedmemCarveoutMaxShared;  // of the kernel that follows, in percent (-1: any)
     uint32_t *map;
     size_t n;
     uint32_t *words[3];
@@ -182,6 +183,7 @@ cudaError_t launch_shoot_split_list(const ShootArgs &a, const int *tiles, int64_
                                     int fma_pairs);
 int fallback_star_split(int64_t nstars);
 cudaError_t launch_bin(const BinArgs &a, cudaStream_t s);  // after launch_clear on the same stream
+int bin_clear_carveout(int64_t n);                         // that clear's carveout for n records
 
 // helpers (api.cu)
 void set_last_error(const std::string &msg);
