@@ -85,8 +85,11 @@ static inline int tile_row_end(const ShootArgs &a, int np, int ty1)
 // do not always spread (440 on 152 SMs: four on some SMs; 256 behind other work on the
 // stream: three), and an SM's reciprocals take the time of all its CTAs.
 // 1e7 stars x 512^2 rays, unsplit (256 CTAs): 981 -> 651 ms;
-// 3000 stars x 704 x 640 rays (440): 334 -> 308 us; other grids of 4 to 576 CTAs and 100 to
-// 200000 stars within 1 % of the same.
+// 3000 stars x 704 x 640 rays (440): 334 -> 308 us.
+// c = 1 leaves room for two: such grids spread by themselves behind a clear of the same
+// carveout (clear.cu), and one CTA keeps an SM less than two thirds busy, which maps on
+// other streams can use.  512 x 256 rays of 3000 stars (128 CTAs), a map on each of four
+// streams 105 -> 83 us a map, on two 108 -> 100, on one 127 either way.
 static cudaError_t spread_smem(int64_t ctas, size_t used, size_t *dyn, size_t *most)
 {
     *dyn = 0;
@@ -99,8 +102,8 @@ static cudaError_t spread_smem(int64_t ctas, size_t used, size_t *dyn, size_t *m
     if (e != cudaSuccess) return e;
     // c of these bytes fit an SM, c + 1 do not
     auto pad = [&](int c) { return (size_t)sm_bytes / (c + 1) + 128 - used - (size_t)reserved; };
-    *dyn = pad((int)((ctas + nsm - 1) / nsm));
-    *most = pad(1);
+    *dyn = pad(ctas <= nsm ? 2 : (int)((ctas + nsm - 1) / nsm));
+    *most = pad(2);
     return cudaSuccess;
 }
 
