@@ -348,8 +348,10 @@ __global__ void __launch_bounds__(kThr) k_disk(const int64_t *__restrict__ P, in
 // neighbouring ones a word, and a thread sums two columns at once (disk_sums): half the
 // loads and additions.  Elsewhere sums are exact in 32 bits, modulo 2^32 in the prefixes,
 // while the largest staged count times |K| is below 2^32 (`limit`; 3.2e6 rays in a pixel for
-// 1317 pixels).  A tile with larger counts takes its sums from the counts' low and high halves
-// in two passes per eight rows, in 64 bits.
+// 1317 pixels).  A tile with larger counts takes the sums modulo 2^32 and, staged once
+// more, those of the counts' high halves, which together give the 64-bit sums: 2048^2 pixels
+// with counts up to 4e6 at R = 20 104.5 us (53 with counts up to 1e5), 201 us in two passes
+// per eight rows, 104.5 us with int64 prefixes; R = 62 623 -> 367 us.
 // Bound by issue slots (77 %) and shared-memory loads (30 words an output at R = 20 pixels
 // packed, 59 not): 4096^2 pixels in 130 us; 164 us unpacked; 373 us with int64 prefixes made
 // by a kernel of their own and staged with their halo (8 bytes a load, three FP64 operations
@@ -493,6 +495,7 @@ __global__ void __launch_bounds__(kThr) k_disk_tile(const uint32_t *__restrict__
     // packed pairs of columns: the segment of a scan is held in registers
     constexpr bool kPacks = kSeg <= 51;
     constexpr int kGroup2 = 2 * kGroup, kPer2 = TY / kGroup2, kRows2 = kPer2 < 8 ? kPer2 : 8;
+    constexpr int kBatches = kPacks ? 1 : kPer / kRows;  // unrolled batches of rows of the unpacked sums
     static_assert(kThr % TX == 0 && kPer % kRows == 0 && kPer2 % kRows2 == 0, "whole batches");
     static_assert(S % 8 == 4, "conflict-free scan");
     constexpr int W = disk_tile_w(TX, S);  // the staged columns start at i0 - W - 1
@@ -634,29 +637,38 @@ __global__ void __launch_bounds__(kThr) k_disk_tile(const uint32_t *__restrict__
             const int c = tid % TX, g = tid / TX, i = i0 + c;
             scan(0, 0xffffffffu);
             const bool large = s_top > limit;
+            // the sums of this thread's rows: modulo 2^32 where they are large, then kept in the
+            // output until those of the counts' high halves complete them
+            // (narrow row strides unrolled ran 3 to 6 % slower, wide ones rolled 2 to 3 %)
+#pragma unroll kBatches
             for (int b = 0; b < kPer; b += kRows) {
                 const int rt = g * kPer + b;
+                if (i >= nx || j0 + rt >= ny) break;
                 uint32_t sum[kRows], lo[kRows], hi[kRows];
-                if (!large) {
-                    if (i < nx && j0 + rt < ny) {
-                        disk_sums<S, W, kRows, false>(T + rt * S + c, B, 0, sum, lo, hi);
+                disk_sums<S, W, kRows, false>(T + rt * S + c, B, 0, sum, lo, hi);
 #pragma unroll
-                        for (int k = 0; k < kRows; ++k)
-                            if (j0 + rt + k < ny) out[(j0 + rt + k) * nx + i] = scale_sum(sum[k], f, fh, fl, fast);
-                    }
-                } else {
-                    uint32_t high[kRows];
-                    stage();
-                    scan(0, 0xffffu);
-                    disk_sums<S, W, kRows, false>(T + rt * S + c, B, 0, sum, lo, hi);
-                    stage();
-                    scan(16, 0xffffu);
+                for (int k = 0; k < kRows; ++k)
+                    if (j0 + rt + k < ny)
+                        out[(j0 + rt + k) * nx + i] =
+                            large ? __uint_as_float(sum[k]) : scale_sum(sum[k], f, fh, fl, fast);
+            }
+            if (large) {
+                stage();
+                scan(16, 0xffffu);
+#pragma unroll kBatches
+                for (int b = 0; b < kPer; b += kRows) {
+                    const int rt = g * kPer + b;
+                    if (i >= nx || j0 + rt >= ny) break;
+                    uint32_t high[kRows], lo[kRows], hi[kRows];
                     disk_sums<S, W, kRows, false>(T + rt * S + c, B, 0, high, lo, hi);
 #pragma unroll
                     for (int k = 0; k < kRows; ++k)
-                        if (i < nx && j0 + rt + k < ny) {
-                            const int64_t t = (int64_t)sum[k] + ((int64_t)high[k] << 16);
-                            out[(j0 + rt + k) * nx + i] = __double2float_rn(__dmul_rn((double)t, f));
+                        if (j0 + rt + k < ny) {
+                            float *dst = out + (j0 + rt + k) * nx + i;
+                            // the low halves add less than 2^32 to high 2^16
+                            const uint64_t from = (uint64_t)high[k] << 16;
+                            const uint64_t t = from + (__float_as_uint(*dst) - (uint32_t)from);
+                            *dst = __double2float_rn(__dmul_rn((double)(int64_t)t, f));
                         }
                 }
             }
