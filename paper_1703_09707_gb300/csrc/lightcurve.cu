@@ -347,7 +347,8 @@ __global__ void __launch_bounds__(kThr) k_disk(const int64_t *__restrict__ P, in
 // Where every staged row's total fits 13 bits the prefixes are kept as 16-bit numbers, two
 // neighbouring ones a word, and a thread sums two columns at once (disk_sums): half the
 // loads and additions.  Elsewhere sums are exact in 32 bits, modulo 2^32 in the prefixes,
-// while the largest staged count times |K| is below 2^32 (`limit`; 3.2e6 rays in a pixel for
+// while the largest staged count times |K|, or the part of K that the
+// map's columns leave, is below 2^32 (`limit`; 3.2e6 rays in a pixel for
 // 1317 pixels).  A tile with larger counts takes the sums modulo 2^32 and, staged once
 // more, those of the counts' high halves, which together give the 64-bit sums: 2048^2 pixels
 // with counts up to 4e6 at R = 20 104.5 us (53 with counts up to 1e5), 201 us in two passes
@@ -827,6 +828,7 @@ struct ConvPlan {
     int Hs = 0;            // disk: support rows |dj| <= Hs
     int Ws = 0;            // disk: the largest half-width, capped at nx
     int64_t count = 0;     // disk: |K|
+    int64_t terms = 0;     // disk: the most pixels of the map that K covers (rows capped at nx)
     DiskGroups groups{};   // disk: runs of support rows of one half-width (capped at nx); n = 0: too many
     size_t off_map = 0;    // workspace offset of the map-sized buffer
     size_t bytes = 0;      // workspace size
@@ -862,6 +864,7 @@ int plan_convolution(const mlens_grid *src, int32_t profile, double size, ConvPl
             const int h = half_width(size, dx, dy, dj);
             if (h >= 0) {
                 count += 2 * (int64_t)h + 1;
+                pl->terms += std::min<int64_t>(2 * (int64_t)h + 1, nx);
                 Hs = std::max(Hs, std::abs(dj));
                 pl->Ws = std::max(pl->Ws, std::min(h, nx));
             }
@@ -953,7 +956,7 @@ cudaError_t launch_disk_tile(const uint32_t *in, int nx, int ny, const ConvPlan 
         }
         *end[kind] = n;
     }
-    const uint32_t limit = (uint32_t)(0xffffffffull / (uint64_t)pl.count);
+    const uint32_t limit = (uint32_t)(0xffffffffull / (uint64_t)pl.terms);
     const bool fast = std::fabs(f) > 0x1p-60 && std::fabs(f) < 0x1p60;
     const float fh = (float)f, fl = (float)(f - (double)fh);
     const dim3 grid((unsigned)((nx + TX - 1) / TX), (unsigned)std::min<int64_t>(((int64_t)ny + TY - 1) / TY, 65535));
@@ -1002,8 +1005,10 @@ int run_convolution(const uint32_t *counts_dev, const mlens_grid *src, int32_t p
         return lc_cuda(e, "cudaDeviceGetAttribute");
     const double f = scale / (double)pl.count;
     // One kernel from the counts wherever a tile fits (sums of 16-bit halves beyond 32
-    // bits need the 64-bit prefixes)
-    if (pl.groups.n > 0 && pl.count <= 65536) {
+    // bits need the 64-bit prefixes).  On maps narrower than the disk only the columns there are
+    // count: 20 x 20000 pixels under a half-width of 3000 and 41 rows 118.9 us with the
+    // 64-bit prefixes -> 24.6 us.
+    if (pl.groups.n > 0 && pl.terms <= 65536) {
         bool done = false;
         if ((int64_t)((nx + 127) / 128) * ((ny + 63) / 64) >= 2 * (int64_t)nsm)
             e = disk_tile_of<128, 64, 140, 172, 204>(counts_dev, nx, ny, pl, f, out_dev, s, kDiskTileSmem3, &done);
