@@ -1331,7 +1331,7 @@ struct LearnSmem {
     __align__(16) TileDesc desc[2];  // this tile's and the next one's
     __align__(16) uint32_t hist[kLearnWin * kLearnWin];  // binning window, cleared as it is flushed
     int win[2];
-    unsigned sred[3];
+    unsigned long long sred[3];
     long long first;
 };
 
@@ -1413,7 +1413,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_shoot_learned(const __grid_cons
     auto desc_of = [&](int64_t item) { return reinterpret_cast<const uint32_t *>(L.desc + (L.items ? L.items[item] : item)); };
     constexpr int kDescWords = sizeof(TileDesc) / 4;
     hist_zero<kLearnWin>(ls.hist);
-    if (tid < 3) ls.sred[tid] = 0u;
+    if (tid < 3) ls.sred[tid] = 0ull;
     int64_t item = blockIdx.x;  // the queue hands out the items from gridDim.x on
     if (tid < kDescWords && item < L.nitems) reinterpret_cast<uint32_t *>(&ls.desc[0])[tid] = desc_of(item)[tid];
     __syncthreads();
@@ -1735,7 +1735,7 @@ __global__ void __launch_bounds__(kThreads, 4) k_shoot_learned(const __grid_cons
         __syncthreads();
         hist_flush<true>(W, a.bin, a.counts);
     }
-    stats_add_block(nb - no - nn, no, nn, ls.sred, a.stats);
+    stats_add_cta(nb - no - nn, no, nn, ls.sred, a.stats);
     if (NET) {
         // a warpgroup that gave up on a wait drains its MMAs (again bounded) before
         // the tensor memory is freed

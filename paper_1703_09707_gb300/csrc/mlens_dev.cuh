@@ -226,4 +226,19 @@ __device__ __forceinline__ void stats_add_block(unsigned binned, unsigned out, u
     }
 }
 
+// The same for the counts of a persistent CTA, which may add up to 2^32 and more over its
+// threads (2^21 tiles of 2048 rays): sums in 64 bits.
+__device__ __forceinline__ void stats_add_cta(unsigned binned, unsigned out, unsigned nan, unsigned long long *sred,
+                                              unsigned long long *stats)
+{
+    const unsigned v[3] = {binned, out, nan};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const unsigned lo = __reduce_add_sync(0xffffffffu, v[k] & 0xffffu), hi = __reduce_add_sync(0xffffffffu, v[k] >> 16);
+        if ((threadIdx.x & 31u) == 0) atomicAdd(&sred[k], ((unsigned long long)hi << 16) + lo);
+    }
+    __syncthreads();
+    if (threadIdx.x < 3 && stats && sred[threadIdx.x]) atomicAdd(&stats[threadIdx.x], sred[threadIdx.x]);
+}
+
 }  // namespace mlens
