@@ -367,7 +367,7 @@ struct DiskGroups {
 // The groups cut into blocks of 8, 4, 2 and 1 rows (integer sums take any order): the
 // stage offset of a block's first row and its half-width; passed by value with
 // the launch and read from the constant bank.
-constexpr int kMaxBlocks = 384;
+constexpr int kMaxBlocks = 384;  // plans of more take the 64-bit prefixes (none that fits a tile's shared memory has as many)
 struct DiskBlocks {
     int n8, n4, n2, n1;  // ends of the blocks of each kind
     int2 at[kMaxBlocks];
@@ -841,6 +841,7 @@ struct ConvPlan {
     int64_t count = 0;     // disk: |K|
     int64_t terms = 0;     // disk: the most pixels of the map that K covers (rows capped at nx)
     DiskGroups groups{};   // disk: runs of support rows of one half-width (capped at nx); n = 0: too many
+    int blocks = 0;        // disk: the blocks of 8, 4, 2 and 1 rows they are cut into (DiskBlocks)
     size_t off_map = 0;    // workspace offset of the map-sized buffer
     size_t bytes = 0;      // workspace size
 };
@@ -894,6 +895,10 @@ int plan_convolution(const mlens_grid *src, int32_t profile, double size, ConvPl
                 G.n = 0;
                 break;
             }
+        }
+        for (int q = 0; q < G.n; ++q) {
+            const int r = G.rows[q];
+            pl->blocks += r / 8 + (r >> 2 & 1) + (r >> 1 & 1) + (r & 1);
         }
         pl->off_map = round256((size_t)(2 * Hs + 1) * sizeof(int));
         pl->bytes = pl->off_map + round256(npix * sizeof(int64_t));
@@ -960,7 +965,6 @@ cudaError_t launch_disk_tile(const uint32_t *in, int nx, int ny, const ConvPlan 
             // 8s first, then at most one block of each smaller kind, from the group's first row on
             const int r0 = m == 8 ? 0 : all / (2 * m) * (2 * m), k = m == 8 ? all / 8 : all / m % 2;
             for (int q = 0; q < k; ++q) {
-                if (n == kMaxBlocks) return cudaErrorInvalidValue;  // the plan has at most kMaxGroups groups: unreachable
                 const int r = (row + r0 + q * m) * S;
                 B.at[n++] = make_int2(r, h);
             }
@@ -1019,7 +1023,7 @@ int run_convolution(const uint32_t *counts_dev, const mlens_grid *src, int32_t p
     // bits need the 64-bit prefixes).  On maps narrower than the disk only the columns there are
     // count: 20 x 20000 pixels under a half-width of 3000 and 41 rows 118.9 us with the
     // 64-bit prefixes -> 24.6 us.
-    if (pl.groups.n > 0 && pl.terms <= 65536) {
+    if (pl.groups.n > 0 && pl.blocks <= kMaxBlocks && pl.terms <= 65536) {
         bool done = false;
         if ((int64_t)((nx + 127) / 128) * ((ny + 63) / 64) >= 2 * (int64_t)nsm)
             e = disk_tile_of<128, 64, 140, 172, 204>(counts_dev, nx, ny, pl, f, out_dev, s, kDiskTileSmem3, &done);
