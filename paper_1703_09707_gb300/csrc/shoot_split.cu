@@ -158,19 +158,22 @@ cudaError_t launch_shoot_split(const ShootArgs &a, int pairs_per_thread, int spl
 
 int auto_star_split(const RayGrid &r, int pairs_per_thread, int64_t nstars, int nsm)
 {
-    // One CTA per SM already keeps the SM's reciprocal unit near its peak, and
-    // a second resident CTA (the kernels are launch-bounded to two per SM)
-    // shares it.  For C = tiles * R equal CTAs of work T / R the map therefore
-    // takes T / R when C <= nsm (one CTA per SM) and about
-    // ceil(C / (2 nsm)) * 2 T / R otherwise (rounds of two CTAs at half speed).
+    // Costs are in whole tiles, two of them an SM's round: C = tiles * R parts of work T / R
+    // take T / R when C <= nsm and ceil(C / (2 nsm)) * 2 T / R otherwise.  The kernels are
+    // finer than that (a tile is two CTAs of half its work, four fit an SM, one alone runs
+    // at four fifths of the SM's rate); the rule keeps to it, since a grid's split decides
+    // beta's last bits, and because what it chooses holds: over 8 to 200 tiles and 4096 to
+    // 65536 stars it takes 0.21 to 0.89 of the unsplit time wherever it splits (76 tiles,
+    // 16384 stars: clusters of 2 548 us, unsplit 689 us).  What it leaves: 40 tiles, 16384
+    // stars 541 us in clusters of 2, 341 us in clusters of 8; 90 tiles, 8192 stars 558 us
+    // unsplit, 341 us in clusters of 8.
     // The split through global memory takes R = the smallest number above
-    // kMaxClusterSplit giving at least 16 CTAs per SM, so the last round is
+    // kMaxClusterSplit giving at least 16 parts per SM, so the last round is
     // nearly full; it is taken if it gains 5 % and leaves every slice
-    // kMinSplitStars stars.  (Cluster splits are not chosen automatically: a
-    // cluster needs all its CTAs free at once within one GPC, and on few-tile
-    // grids that fragmentation cost as much as the split gained.)  With too few
-    // stars for that many slices, the clusters of 2, 4 or 8 CTAs are weighed the
-    // same way.
+    // kMinSplitStars stars: its CTAs start one at a time, where a cluster needs all its
+    // CTAs free at once within one GPC (1e7 stars, 128 tiles: 518 ms, clusters of 8 541 ms,
+    // unsplit 651 ms).  With too few stars for that many slices, the clusters of 2, 4 or 8
+    // CTAs are weighed the same way.
     const double tiles = (double)tiles_of(r, pairs_per_thread);
     const double sms = (double)(nsm > 0 ? nsm : 1);
     auto cost = [&](int64_t R) {
