@@ -103,8 +103,8 @@ int mlens_set_precision(mlens_ctx *ctx, int32_t precision);
 
 /*
  * mlens_set_tuning -- launch shape of the FP32 kernels for later calls on this
- * context: rays_per_thread in {4, 8} (tile 64 x 16 or 64 x 32 rays per CTA of
- * 256 threads), star_stage in {128, 256, 512} stars staged through shared
+ * context: rays_per_thread in {4, 8} (tile 64 x 16 or 64 x 32 rays, two CTAs of
+ * 128 threads), star_stage in {128, 256, 512} stars staged through shared
  * memory at a time (0 = 256; the kernels now stage 128 whatever the setting, which
  * still decides whether the star sum may be split), and fma_pairs in {0, 1}: 0 takes every
  * reciprocal 1/r^2 from the MUFU unit (16 per SM per clock, the bound of the

@@ -1316,7 +1316,12 @@ cudaError_t ff_cell_rec(const float *coef, const float *sc, const float *ec, int
     return cudaGetLastError();
 }
 
-constexpr int kLearnWin = 32;  // a learned tile's rays land on a patch of about 12 x 6 pixels
+// Binning window: a learned tile's rays land on a patch of about 12 x 6 pixels of a 4096^2 map;
+// on maps of finer pixels the rays outside it take global atomics.  2e5 stars, order-16 series
+// (2.7e8 rays) into 2048^2, 8192^2, 16384^2 and 24576^2 pixels: 1.90, 2.11, 2.78 and 3.76 ms; with
+// a window of 64, cleared and flushed whole by every tile of the former kernel, 2.96, 3.08,
+// 3.40 and 4.02 ms.  (64 would leave room for three CTAs an SM beside the network's operands.)
+constexpr int kLearnWin = 32;
 struct LearnSmem {
     __align__(128) unsigned char w2cm[kHid * kHid * 2];  // W2 / 2 [out][in], BF16, core-matrix layout (B operand)
     uint64_t mbar[2];     // per warpgroup: completion of its tensor-core MMAs
@@ -1768,8 +1773,9 @@ cudaError_t ff_learned_grid(int *grid)
     // The persistent grid takes the resident CTAs per SM of the kernel without
     // tensor-core code (four: launch-bounded to 64 registers per thread).  The
     // tensor-core variant has the same register limit and fits four CTAs in shared
-    // and tensor memory, though the occupancy query has reported fewer for it; CTAs
-    // beyond those resident only find the shared work queue empty.
+    // and tensor memory, though the occupancy query has reported fewer for it.  Every CTA
+    // owns the item of its number, so one beyond those resident would still work off that
+    // tile after another CTA has ended.
     int per_sm = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_shoot_learned<false, false>, kThreads,
                                                                   sizeof(NearStage));

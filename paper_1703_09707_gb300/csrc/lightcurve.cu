@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(kThr) k_disk(const int64_t *__restrict__ P, in
 // The row stride S is a template parameter, so that the rows' loads have immediate
 // addresses; S = 4 x odd, four segments of S / 4 words: the scan's 8 rows x 4 segments
 // per warp fall on 32 different banks.
-// Where every staged row's total fits 13 bits the prefixes are kept as 16-bit numbers, two
+// Where every staged row's total fits 13 bits (47 rays a pixel at R = 20 pixels) the prefixes are kept as 16-bit numbers, two
 // neighbouring ones a word, and a thread sums two columns at once (disk_sums): half the
 // loads and additions.  Elsewhere sums are exact in 32 bits, modulo 2^32 in the prefixes,
 // while the largest staged count times |K|, or the part of K that the
@@ -981,7 +981,10 @@ cudaError_t launch_disk_tile(const uint32_t *in, int nx, int ny, const ConvPlan 
 
 // The disk in one kernel: 128 x 64 outputs (the least halo) where three CTAs fit an SM
 // and the tiles fill the SMs twice, else 64 x 64 where they fill them once, else 64 x 32; the
-// smallest row stride with room for the support.  *done = false: no tile fits its shared memory.
+// smallest row stride with room for the support.  *done = false: no tile fits its shared memory,
+// or the support is wider than the longest row (half-width 117).  Such supports of few rows
+// (pixels much higher than wide) take the int64 prefixes, which there are faster than the tiles of int64
+// prefixes that took them before: 4096^2 pixels, half-width 145, five rows 280 -> 194 us.
 template <int TX, int TY, int S, int... More>
 cudaError_t disk_tile_of(const uint32_t *in, int nx, int ny, const ConvPlan &pl, double f, float *out, cudaStream_t s,
                          size_t most, bool *done)

@@ -130,8 +130,8 @@ __device__ __forceinline__ int pair_axis_rough(float bh, const AxisPair &A)
 // them land in a small patch of the source map.  The CTA counts that patch in
 // a W x W shared-memory window (placed around the pixel of one of its rays, inside the
 // map) and adds the window to the global map at the end; rays outside the window go
-// straight to global atomics.  W is 64, or 32 for the direct sum's half tiles.  One atomic
-// per ray: the shared-memory increment merges a warp's equal pixels in hardware, which
+// straight to global atomics.  W is 64, or 32 for the direct sum's half tiles and the
+// learned tiles.  One atomic per ray: the shared-memory increment merges a warp's equal pixels in hardware, which
 // cost less than finding runs of equal pixels with a shuffle, a vote and a branch per ray.
 constexpr int kWin = 64;
 
