@@ -1383,7 +1383,8 @@ __device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
 // Four CTAs per SM (64 registers, spills included; tensor memory holds four CTAs' 128
 // columns): eight warps per scheduler hide the latency of the 128 hardware tanh per ray.
 // Three CTAs: 42.9 and 1.95 ms for the two maps below.
-// Bound with the network by MUFU (132 results a ray; 72 % busy), without it by issue slots.
+// Bound with the network by MUFU (132 results a ray; 70 % busy, the threads waiting for its
+// results and at the tile's barriers), without it by issue slots.
 // 32768 x 33024 rays of 1e6 stars, no cell flagged: 44.3 -> 41.1 ms; 2.7e8 rays, order-16
 // series alone, 2.47 -> 1.92 ms: descriptors and records from the fit, the next tile
 // fetched ahead, one window clear and four barriers less a tile, near stars without
